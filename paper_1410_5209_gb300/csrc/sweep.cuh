@@ -249,20 +249,21 @@ struct PredictArgs {
     const int32_t *coords;
     T *out;
     DeviceStatus *stat;
+    float big;  // float contexts: values from here on take the FP64 form (launch_predict)
 };
 template <class T>
 void launch_predict(const PredictArgs<T> &a, cudaStream_t st);
 // Tiled fold-in (K < 128): block table of a batch of requests (offsets[n_req + 1] into
-// the concatenated entries; 256 entries per block), partial buffer length, launch.
+// the concatenated entries), partial buffer length, launch.
 bool foldin_tiled_ok(int K);
 int foldin_plan_blocks(const int64_t *offsets, int n_req, std::vector<int64_t> &blk_range,
                        std::vector<int32_t> &blk_req, std::vector<int32_t> &req_blk);
 size_t foldin_part_elems(int K, int blocks);
 // Refinement buffers of a tiled fold-in: returns the FP64 partial residual elements
-// (blocks x K); *fac_elems receives the factor store's elements (n_req x K(K+1)/2).
+// (blocks x K); *fac_elems receives the factor store's elements.
 size_t foldin_refine_elems(int K, int blocks, int n_req, size_t *fac_elems);
 template <class T>
-void launch_foldin_tiled(const FoldArgs<T> &a, int blocks, int n_req, cudaStream_t st);
+void launch_foldin_tiled(const FoldArgs<T> &a, int blocks, cudaStream_t st);
 template <class T>
 size_t foldin_smem_bytes(int K);
 
