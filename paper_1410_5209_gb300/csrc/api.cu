@@ -1832,9 +1832,10 @@ struct Impl : CtxBase {
             f_fac.ensure(fac_elems, st);
         }
         // one int64 staging buffer: block entry ranges [2B], then as int32 the blocks'
-        // requests [B], the requests' first blocks [n_req + 1] and their status [n_req]
+        // requests [B], the requests' first blocks [n_req + 1], their status [n_req] and two
+        // counts of finished blocks [2 n_req]
         const size_t B = (size_t)std::max(blocks, 1);
-        const size_t n32 = B + 2 * (size_t)n_req + 1;
+        const size_t n32 = B + 4 * (size_t)n_req + 1;
         const size_t n64 = 2 * B + (n32 + 1) / 2;
         f_meta.ensure(n64, st);
         std::vector<int64_t> meta(n64, 0);
@@ -1842,8 +1843,6 @@ struct Impl : CtxBase {
         int32_t *m32 = reinterpret_cast<int32_t *>(meta.data() + 2 * B);
         std::copy(blk_req.begin(), blk_req.end(), m32);
         std::copy(req_blk.begin(), req_blk.end(), m32 + B);
-        int32_t *st_host = m32 + B + n_req + 1;
-        std::fill(st_host, st_host + n_req, 0);
         if (m > 0) {
             TFS_CUDA(cudaMemcpyAsync(f_other.p, other, (size_t)m * (N - 1) * sizeof(int32_t),
                                      cudaMemcpyHostToDevice, st));
@@ -1870,11 +1869,13 @@ struct Impl : CtxBase {
         a.blk_range = f_meta.p;
         a.blk_req = d32;
         a.req_blk = d32 + B;
+        a.n_req = n_req;
         a.req_status = const_cast<int32_t *>(d32 + B + n_req + 1);
+        a.req_count = a.req_status + n_req;
         a.refine = refine ? 1 : 0;
         a.fac = refine ? f_fac.p : nullptr;
         a.rpart = refine ? f_rpart.p : nullptr;
-        launch_foldin_tiled<T>(a, blocks, n_req, st);
+        launch_foldin_tiled<T>(a, blocks, st);
         std::vector<T> rows((size_t)n_req * K);
         TFS_CUDA(cudaMemcpyAsync(status, a.req_status, (size_t)n_req * sizeof(int32_t),
                                  cudaMemcpyDeviceToHost, st));

@@ -117,19 +117,22 @@ struct FoldArgs {
     T lambda;
     T *out;
     DeviceStatus *stat;
-    T *part;      // [blocks][K (K + 1) / 2 + K] partial Gram / rhs of the tiled fold-in
+    T *part;      // [blocks] partial Gram / rhs tiles of the tiled fold-in
     // tiled fold-in of a batch: per block its entry range and request, per request its
-    // first block (n_req + 1), per request a status word (1 bad index, 2 bad pivot);
-    // out is then [n_req][K]
+    // first block (n_req + 1), a status word (1 bad index, 2 bad pivot) and two counts of
+    // finished blocks (req_count [2][n_req], zero on entry); out is then [n_req][K]
+    int n_req;
     const int64_t *blk_range;
     const int32_t *blk_req;
     const int32_t *req_blk;
     int32_t *req_status;
+    int32_t *req_count;
     // float contexts: one step of iterative refinement of every request's solve.  The
-    // solve keeps its Cholesky factor in fac [n_req][K (K + 1) / 2]; a second pass over
-    // the request's entries forms the residual of the normal equations,
-    // c - (B + lambda I) x0 = sum_e h_e (x_e - h_e . x0) - lambda x0, in FP64 (per-block
-    // partials in rpart [blocks][K]); the correction solved with the factor is added.
+    // solve keeps its Cholesky factor in fac [n_req] (rows of K rounded up to 4); a second
+    // pass over the request's entries forms the residual of the normal equations,
+    // c - (B + lambda I) x0 = sum_e h_e (x_e - h_e . x0) - lambda x0, to twice the working
+    // precision (per-block partials in rpart [blocks][K], FP64); the correction solved with
+    // the factor is added.
     int refine;
     T *fac;
     double *rpart;
