@@ -196,6 +196,7 @@ struct ModeLayout {
     Buf<int32_t> id_of;     // degree rank -> row id
     Buf<int32_t> groups;    // slot groups of split rows (first slot, count), wide subsets
     int n_groups = 0;
+    int n_light = 0;  // split rows of at most kLightSlots slots: the first of `split`
     std::vector<int64_t> deg_cum;  // host: entries of the first R rows in degree-rank order
     // per bin, the step units and entries of the bins before it (gather-plan regions)
     Buf<uint32_t> plan_base;  // [2 (P + 1)]
@@ -392,6 +393,7 @@ struct Impl : CtxBase {
         std::vector<int64_t> bin_ptr;
         std::vector<SplitRow> split, single;
         std::vector<int32_t> groups;  // slot groups of rows with many chunks (wide subsets)
+        int n_light = 0;  // split rows of at most kLightSlots slots: the first of `split`
         int64_t n_slots = 0;
         // gather-plan regions: step units (max(1, ceil(len / 32)) per item) and entries
         // of the bins before each bin, [P + 1] each
@@ -866,7 +868,6 @@ struct Impl : CtxBase {
         tf_status s = plan_mode(off.data(), I, P, 0, policy, seed, h.items, h.n_slots, h.bin_ptr);
         if (s != TF_OK) throw ApiError{s, "row scheduling failed"};
         // rows and their slots (a row's slots are consecutive, in entry order):
-        // single-item rows are solved by k_solve_rows, split rows by k_combine
         std::vector<int32_t> item_of_slot((size_t)h.n_slots, -1);
         for (size_t i = 0; i < h.items.size(); ++i) item_of_slot[(size_t)h.items[i].slot] = (int32_t)i;
         for (int64_t q = 0; q < h.n_slots;) {
@@ -878,6 +879,11 @@ struct Impl : CtxBase {
             (q2 - q > 1 ? h.split : h.single).push_back(sr);
             q = q2;
         }
+        h.n_light = (int)(std::stable_partition(h.split.begin(), h.split.end(),
+                                                [](const SplitRow &r) {
+                                                    return r.n_slots <= kLightSlots;
+                                                }) -
+                          h.split.begin());
         for (const SplitRow &sr : h.split)
             if (sr.n_slots > kSlotGroup)
                 for (int g = 0; g < sr.n_slots; g += kSlotGroup) {
@@ -921,6 +927,7 @@ struct Impl : CtxBase {
         L.single.alloc(h.single.size(), st);
         L.n_groups = (int)(h.groups.size() / 2);
         L.groups.alloc(std::max<size_t>(h.groups.size(), 2), st);
+        L.n_light = h.n_light;
         L.plan_base.alloc(h.plan_base.size(), st);
         L.plan_units = h.plan_units;
         stage.copy(L.groups.p, h.groups.data(), h.groups.size() * sizeof(int32_t), st);
@@ -1214,6 +1221,7 @@ struct Impl : CtxBase {
                 pk.off_prev = off_prev;
                 pk.S = Sp;
                 pk.Q = Qp;
+                pk.prev_in_cur = s > 0;
                 timed(TF_KIND_PACK, [&] { launch_pack<T>(pk, st); });
                 ++launches;
                 if (bf16_rows) {
@@ -1359,16 +1367,12 @@ struct Impl : CtxBase {
                     }
                         ++launches;
                     solved:
-                        if (L.n_single > 0) {
-                            timed(TF_KIND_SOLVE,
-                                  [&] { launch_solve_rows<T>(a, CM, L.single.p, L.n_single, st); });
-                            ++launches;
-                        }
-                        if (L.n_split > 0) {
-                            timed(TF_KIND_COMBINE,
-                                  [&] { launch_combine<T>(a, CM, L.split.p, L.n_split, st); });
-                            ++launches;
-                        }
+                        timed(TF_KIND_SOLVE, [&] {
+                            const SolveRows rows{L.single.p, L.split.p, L.n_single, L.n_light,
+                                                 L.n_split - L.n_light};
+                            launch_solve_rows<T>(a, CM, rows, st);
+                        });
+                        ++launches;
                         if (bf16_rows) {  // the rows just solved, into the bfloat16 copy
                             timed(TF_KIND_PACK, [&] {
                                 launch_slice_bf16((const float *)Z[n].p, Zb[n].p, dims[n], W, Wb,

@@ -12,11 +12,10 @@
 //      from shared memory, refreshes its residual copy to this split's R-hat on the
 //      first inner iteration (Algorithm 1; done lazily per copy, see PassArgs) and
 //      accumulates B += h h^T (lower triangle) and c += r_hat h in registers.
-// The warp then sums B and c with butterfly shuffles.  A whole row is solved right
-// there: B + lambda I_C (lambda * |Omega_i| when weighted) by a register Cholesky
-// (Section 3.1), and the new C parameters go to the packed slice and to A^(n).  A chunk
-// writes its partial (B, c) to its slot instead; k_combine sums the slots of each
-// split row in slot order (deterministic) and solves.
+// The warp then sums B and c with butterfly shuffles and writes them to the item's slot.
+// k_solve_rows sums the slots of each row in a fixed order and solves B + lambda I_C (lambda
+// * |Omega_i| when weighted) by a register Cholesky (Section 3.1); the new C parameters go to
+// the packed slice and to A^(n).
 #pragma once
 
 #include <algorithm>
@@ -86,11 +85,26 @@ __device__ __forceinline__ T warp_sum(T v) {
     return v;
 }
 
+// How the Cholesky keeps its pivots and divides by them.  Double: inverted once per column,
+// since an FP64 division is a dozen instructions of the FP64 unit, which issues a warp's
+// instruction over 64 cycles.  Float: the square root and true divisions (the rounding of
+// every float row stays that of the plain formula).
+template <class T>
+__device__ __forceinline__ T chol_pivot(T root) {
+    if constexpr (sizeof(T) == 8) return T(1) / root;
+    return root;
+}
+template <class T>
+__device__ __forceinline__ T chol_over(T v, T pivot) {
+    if constexpr (sizeof(T) == 8) return v * pivot;
+    return v / pivot;
+}
+
 // Cholesky factor, in place, of B + lam I for the leading C x C block of a CM x CM packed
-// lower triangle; rows/columns >= C are replaced by the identity.  min_ratio receives the
-// smallest pivot ratio d_j / (B_jj + lam) over the leading block (1 when perfectly
-// conditioned, near 0 when a column is nearly a combination of the earlier ones).
-// Returns false when a pivot is <= 0.
+// lower triangle; rows/columns >= C are replaced by the identity.  The diagonal holds
+// chol_pivot(L_jj).  min_ratio receives the smallest pivot ratio d_j / (B_jj + lam) over the
+// leading block (1 when perfectly conditioned, near 0 when a column is nearly a combination
+// of the earlier ones).  Returns false when a pivot is <= 0.
 template <class T, int CM>
 __device__ __forceinline__ bool chol_factor(T (&B)[CM * (CM + 1) / 2], int C, T lam,
                                             T &min_ratio) {
@@ -108,22 +122,27 @@ __device__ __forceinline__ bool chol_factor(T (&B)[CM * (CM + 1) / 2], int C, T 
     }
     bool ok = true;
     min_ratio = T(1);
+    // (trip counts independent of the outer index: with triangular loops the compiler left
+    // the matrix of CM = 6 and 8 in local memory)
 #pragma unroll
     for (int j = 0; j < CM; ++j) {
         const T a_jj = B[tri(j, j)];
         T d = a_jj;
 #pragma unroll
-        for (int k = 0; k < j; ++k) d -= B[tri(j, k)] * B[tri(j, k)];
+        for (int k = 0; k < CM; ++k)
+            if (k < j) d -= B[tri(j, k)] * B[tri(j, k)];
         ok = ok && (d > T(0));
         if (a_jj > T(0)) min_ratio = fmin(min_ratio, d / a_jj);
-        const T ljj = sqrt(d > T(0) ? d : T(1));
-        B[tri(j, j)] = ljj;
+        const T piv = chol_pivot<T>(sqrt(d > T(0) ? d : T(1)));
+        B[tri(j, j)] = piv;
 #pragma unroll
-        for (int i = j + 1; i < CM; ++i) {
+        for (int i = 0; i < CM; ++i) {
+            if (i <= j) continue;
             T s = B[tri(i, j)];
 #pragma unroll
-            for (int k = 0; k < j; ++k) s -= B[tri(i, k)] * B[tri(j, k)];
-            B[tri(i, j)] = s / ljj;
+            for (int k = 0; k < CM; ++k)
+                if (k < j) s -= B[tri(i, k)] * B[tri(j, k)];
+            B[tri(i, j)] = chol_over<T>(s, piv);
         }
     }
     return ok;
@@ -139,14 +158,14 @@ __device__ __forceinline__ void chol_apply(const T (&L)[CM * (CM + 1) / 2], cons
         T s = (i < C) ? r[i] : T(0);
 #pragma unroll
         for (int k = 0; k < i; ++k) s -= L[tri(i, k)] * y[k];
-        y[i] = s / L[tri(i, i)];
+        y[i] = chol_over<T>(s, L[tri(i, i)]);
     }
 #pragma unroll
     for (int i = CM - 1; i >= 0; --i) {
         T s = y[i];
 #pragma unroll
         for (int k = i + 1; k < CM; ++k) s -= L[tri(k, i)] * x[k];
-        x[i] = s / L[tri(i, i)];
+        x[i] = chol_over<T>(s, L[tri(i, i)]);
     }
 }
 
@@ -453,8 +472,7 @@ __device__ __forceinline__ int run_head(uint32_t heads, int lane) {
 }
 
 // End of an item: warp-sum (B, c) with butterflies and store them in the item's
-// partial slot (the solves run afterwards, all rows in parallel: k_solve_rows /
-// k_combine).  Lane k stores values k, k + 32, ...; the summation order is fixed.
+// partial slot (the solves run afterwards, all rows in parallel: k_solve_rows).  Lane k stores values k, k + 32, ...; the summation order is fixed.
 template <class T, int CM>
 __device__ __forceinline__ void finish_item(const PassArgs<T> &a, const Step &s,
                                             T (&Bacc)[CM * (CM + 1) / 2], T (&cacc)[CM],
@@ -762,23 +780,30 @@ __global__ void __launch_bounds__(pass_max_warps<T, CM>() * kWarp, 1)
     }
 }
 
-// Rows held by a single item: one thread per row reads its slot and solves
-// (B + lambda I) a = c (Eq. 4) by the register Cholesky of Section 3.1.
+// Row solves of a mode: (B + lambda I) a = c (Eq. 4) for every row, by the register Cholesky
+// of Section 3.1 with one lane per row, in one launch.
+//   Light rows (up to kLightSlots partial slots): a warp takes 32 of them.  It sums the
+//   rows' slots into shared memory with consecutive lanes on consecutive values, up to 24
+//   loads in flight per lane, and each lane then solves its row.
+//   Heavy rows: one block each; thread (g, v) adds value v of every G-th slot from g on
+//   (eight loads in flight), the G sums are added in order, one lane solves.
+// Bound: latency, reading the slots (C = 10: 260 B a row) and the scattered columns of the
+// factor rows written (one 32-byte sector per value where K is large).  Before, one launch
+// solved the single-slot rows, each thread reading its row's slot at a stride of NB values,
+// and a second took 512 threads per split row: 44 + 55 us per mode of 1e5 rows (1e8 entries,
+// C = 10), now 70; 1,000 FP64 rows of two slots, C = 5: 127 us (a lone lane's FP64
+// instructions take the unit as long as a full warp's), now 25.
 // XS: the solve options of float contexts (refinement / FP64 fallback) are on; the plain
 // Cholesky otherwise, so that the default kernels carry none of their registers.
 template <class T, int CM, bool XS>
-__global__ void __launch_bounds__(128) k_solve_rows(const PassArgs<T> a, const SplitRow *rows,
-                                                    int n_rows) {
-    constexpr int NT = CM * (CM + 1) / 2, NB = NT + CM;
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n_rows) return;
-    const SplitRow sr = rows[r];
-    const T *p = a.partials + (int64_t)sr.first_slot * NB;
+__device__ __forceinline__ void solve_and_write(const PassArgs<T> &a, const SplitRow &sr,
+                                                const T *sum) {
+    constexpr int NT = CM * (CM + 1) / 2;
     T B[NT], c[CM], x[CM];
 #pragma unroll
-    for (int q = 0; q < NT; ++q) B[q] = p[q];
+    for (int q = 0; q < NT; ++q) B[q] = sum[q];
 #pragma unroll
-    for (int q = 0; q < CM; ++q) c[q] = p[NT + q];
+    for (int q = 0; q < CM; ++q) c[q] = sum[NT + q];
     const T lam = a.weighted ? a.lambda * (T)sr.len : a.lambda;
     if (XS ? row_solve<T, CM>(a, B, c, lam, x) : chol_solve<T, CM>(B, c, a.C, lam, x))
         write_row<T, CM>(a, sr.row, x);
@@ -786,40 +811,92 @@ __global__ void __launch_bounds__(128) k_solve_rows(const PassArgs<T> a, const S
         atomicAdd(&a.stat->singular_rows, 1ull);
 }
 
-template <class T, int CM, bool XS>
-__global__ void __launch_bounds__(kCombineThreads) k_combine(const PassArgs<T> a,
-                                                             const SplitRow *rows) {
-    constexpr int NT = CM * (CM + 1) / 2, NB = NT + CM;
-    constexpr int G = kCombineThreads / NB;
-    __shared__ T red[G * NB];
-    __shared__ T tot[NB];
-    const SplitRow sr = rows[blockIdx.x];
-    const int t = threadIdx.x, g = t / NB, v = t - g * NB;
-    if (g < G) {
+constexpr int kSolveThreads = 128;
+
+// Sum of a heavy row's slots at p into tot[NB]; red: G * NB values (both shared memory).
+template <class T, int NB>
+__device__ __forceinline__ void sum_slots(const T *p, int count, T *red, T *tot) {
+    constexpr int G = kSlotSums / NB, U = 8;
+    const int tid = threadIdx.x;
+    for (int t = tid; t < G * NB; t += kSolveThreads) {
+        const int g = t / NB, v = t - g * NB;
         T s = T(0);
-        for (int k = g; k < sr.n_slots; k += G)
-            s += a.partials[(int64_t)(sr.first_slot + k) * NB + v];
+        for (int k = g; k < count; k += U * G) {
+            T w[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) w[u] = k + u * G < count ? p[(int64_t)(k + u * G) * NB + v] : T(0);
+#pragma unroll
+            for (int u = 0; u < U; ++u) s += w[u];
+        }
         red[t] = s;
     }
     __syncthreads();
-    if (t < NB) {
+    for (int v = tid; v < NB; v += kSolveThreads) {
         T s = T(0);
-        for (int gg = 0; gg < G; ++gg) s += red[gg * NB + t];
-        tot[t] = s;
+        for (int g = 0; g < G; ++g) s += red[g * NB + v];
+        tot[v] = s;
     }
     __syncthreads();
-    if (t == 0) {
-        T B[NT], c[CM], x[CM];
-#pragma unroll
-        for (int q = 0; q < NT; ++q) B[q] = tot[q];
-#pragma unroll
-        for (int q = 0; q < CM; ++q) c[q] = tot[NT + q];
-        const T lam = a.weighted ? a.lambda * (T)sr.len : a.lambda;
-        if (XS ? row_solve<T, CM>(a, B, c, lam, x) : chol_solve<T, CM>(B, c, a.C, lam, x))
-            write_row<T, CM>(a, sr.row, x);
-        else
-            atomicAdd(&a.stat->singular_rows, 1ull);
+}
+
+// A warp's 32 rows of sums (odd stride: lanes reading their rows do not conflict), or a
+// heavy row's group sums and total.
+template <class T, int CM>
+constexpr size_t solve_rows_smem() {
+    constexpr int NB = CM * (CM + 1) / 2 + CM;
+    constexpr int light = kSolveThreads * (NB | 1), heavy = kSlotSums + NB;
+    return sizeof(T) * (size_t)(light > heavy ? light : heavy);
+}
+
+template <class T, int CM, bool XS>
+__global__ void __launch_bounds__(kSolveThreads) k_solve_rows(const PassArgs<T> a,
+                                                              const SolveRows r) {
+    constexpr int NT = CM * (CM + 1) / 2, NB = NT + CM, NBP = NB | 1;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T *sm = reinterpret_cast<T *>(smem_raw);
+    if ((int)blockIdx.x < r.n_heavy) {  // first, the longest
+        const SplitRow sr = r.split[r.n_light + blockIdx.x];
+        T *tot = sm + kSlotSums;
+        sum_slots<T, NB>(a.partials + (int64_t)sr.first_slot * NB, sr.n_slots, sm, tot);
+        if (threadIdx.x == 0) solve_and_write<T, CM, XS>(a, sr, tot);
+        return;
     }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i = ((int)blockIdx.x - r.n_heavy) * kSolveThreads + (int)threadIdx.x;
+    SplitRow sr{};
+    if (i < r.n_single)
+        sr = r.single[i];
+    else if (i < r.n_single + r.n_light)
+        sr = r.split[i - r.n_single];
+    T *buf = sm + warp * 32 * NBP;
+    constexpr int U = 8;
+    const bool one = __all_sync(0xFFFFFFFFu, sr.n_slots <= 1);
+    for (int q0 = lane; q0 < 32 * NB; q0 += 32 * U) {
+        T s[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int q = q0 + 32 * u, w = q / NB, v = q - w * NB;
+            const int first = __shfl_sync(0xFFFFFFFFu, sr.first_slot, w & 31);
+            const int n = __shfl_sync(0xFFFFFFFFu, sr.n_slots, w & 31);
+            const T *p = a.partials + (int64_t)first * NB + v;
+            const int ns = q < 32 * NB ? n : 0;
+            s[u] = ns > 0 ? p[0] : T(0);
+            if (!one) {
+                T t[kLightSlots];
+#pragma unroll
+                for (int k = 1; k < kLightSlots; ++k) t[k] = k < ns ? p[k * NB] : T(0);
+#pragma unroll
+                for (int k = 1; k < kLightSlots; ++k) s[u] += t[k];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int q = q0 + 32 * u, w = q / NB, v = q - w * NB;
+            if (q < 32 * NB) buf[w * NBP + v] = s[u];
+        }
+    }
+    __syncwarp();
+    if (sr.n_slots > 0) solve_and_write<T, CM, XS>(a, sr, buf + lane * NBP);
 }
 
 // Residual of copy n against the columns held in the slices' "cur" region (the last
@@ -961,23 +1038,15 @@ void launch_mode_pass_cm(const PassArgs<T> &a, const PassPlan &plan, cudaStream_
 }
 
 template <class T, int CM>
-void launch_combine_cm(const PassArgs<T> &a, const SplitRow *rows, int n_rows, cudaStream_t st) {
-    if (n_rows <= 0) return;
-    if (sizeof(T) == 4 && (a.refine || a.cond_limit > 0.f))
-        k_combine<T, CM, true><<<n_rows, kCombineThreads, 0, st>>>(a, rows);
-    else
-        k_combine<T, CM, false><<<n_rows, kCombineThreads, 0, st>>>(a, rows);
-    TFS_CUDA(cudaGetLastError());
-}
-
-template <class T, int CM>
-void launch_solve_rows_cm(const PassArgs<T> &a, const SplitRow *rows, int n_rows,
-                          cudaStream_t st) {
-    if (n_rows <= 0) return;
-    if (sizeof(T) == 4 && (a.refine || a.cond_limit > 0.f))
-        k_solve_rows<T, CM, true><<<(n_rows + 127) / 128, 128, 0, st>>>(a, rows, n_rows);
-    else
-        k_solve_rows<T, CM, false><<<(n_rows + 127) / 128, 128, 0, st>>>(a, rows, n_rows);
+void launch_solve_rows_cm(const PassArgs<T> &a, const SolveRows &r, cudaStream_t st) {
+    const int64_t blocks =
+        r.n_heavy + ((int64_t)r.n_single + r.n_light + kSolveThreads - 1) / kSolveThreads;
+    if (blocks <= 0) return;
+    const bool xs = sizeof(T) == 4 && (a.refine || a.cond_limit > 0.f);
+    auto kern = xs ? k_solve_rows<T, CM, true> : k_solve_rows<T, CM, false>;
+    constexpr size_t smem = solve_rows_smem<T, CM>();
+    TFS_CUDA(raise_smem_limit((const void *)kern, (int)smem));
+    kern<<<(unsigned)blocks, kSolveThreads, smem, st>>>(a, r);
     TFS_CUDA(cudaGetLastError());
 }
 
@@ -1031,27 +1100,11 @@ PassPlan mode_pass_plan_impl(int CM, int N, int n, bool first, int num_sms, int 
 }
 
 template <class T>
-void launch_combine_impl(const PassArgs<T> &a, int CM, const SplitRow *rows, int n_rows,
-                         cudaStream_t st) {
+void launch_solve_rows_impl(const PassArgs<T> &a, int CM, const SolveRows &r, cudaStream_t st) {
     switch (CM) {
-#define TFS_CASE(cm)                                   \
-    case cm:                                           \
-        launch_combine_cm<T, cm>(a, rows, n_rows, st); \
-        return;
-        TFS_FOR_EACH_CM(TFS_CASE)
-#undef TFS_CASE
-        default:
-            throw ApiError{TF_EINVAL, "no combine instance for this C"};
-    }
-}
-
-template <class T>
-void launch_solve_rows_impl(const PassArgs<T> &a, int CM, const SplitRow *rows, int n_rows,
-                            cudaStream_t st) {
-    switch (CM) {
-#define TFS_CASE(cm)                                       \
-    case cm:                                               \
-        launch_solve_rows_cm<T, cm>(a, rows, n_rows, st);  \
+#define TFS_CASE(cm)                             \
+    case cm:                                     \
+        launch_solve_rows_cm<T, cm>(a, r, st);   \
         return;
         TFS_FOR_EACH_CM(TFS_CASE)
 #undef TFS_CASE

@@ -1,4 +1,4 @@
-// Instantiation of the mode-pass and combine kernels for float (one translation unit
+// Instantiation of the mode-pass and row-solve kernels for float (one translation unit
 // per element type, so the two compile in parallel).
 #include <string.h>
 
@@ -22,20 +22,13 @@ int res_grid<float>(int CM, int P, int N) {
 }
 
 template <>
-void launch_combine<float>(const PassArgs<float> &a, int CM, const SplitRow *rows, int n_rows,
-                          cudaStream_t st) {
-    launch_combine_impl<float>(a, CM, rows, n_rows, st);
-}
-
-template <>
 void launch_res<float>(const ResArgs<float> &a, int CM, cudaStream_t st) {
     launch_res_impl<float>(a, CM, st);
 }
 
 template <>
-void launch_solve_rows<float>(const PassArgs<float> &a, int CM, const SplitRow *rows, int n_rows,
-                            cudaStream_t st) {
-    launch_solve_rows_impl<float>(a, CM, rows, n_rows, st);
+void launch_solve_rows<float>(const PassArgs<float> &a, int CM, const SolveRows &r, cudaStream_t st) {
+    launch_solve_rows_impl<float>(a, CM, r, st);
 }
 
 bool tma_pass_supported(int CM, int N) {

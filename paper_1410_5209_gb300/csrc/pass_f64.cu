@@ -1,4 +1,4 @@
-// Instantiation of the mode-pass and combine kernels for double (one translation unit
+// Instantiation of the mode-pass and row-solve kernels for double (one translation unit
 // per element type, so the two compile in parallel).
 #include "mode_pass.cuh"
 
@@ -20,20 +20,13 @@ int res_grid<double>(int CM, int P, int N) {
 }
 
 template <>
-void launch_combine<double>(const PassArgs<double> &a, int CM, const SplitRow *rows, int n_rows,
-                          cudaStream_t st) {
-    launch_combine_impl<double>(a, CM, rows, n_rows, st);
-}
-
-template <>
 void launch_res<double>(const ResArgs<double> &a, int CM, cudaStream_t st) {
     launch_res_impl<double>(a, CM, st);
 }
 
 template <>
-void launch_solve_rows<double>(const PassArgs<double> &a, int CM, const SplitRow *rows, int n_rows,
-                            cudaStream_t st) {
-    launch_solve_rows_impl<double>(a, CM, rows, n_rows, st);
+void launch_solve_rows<double>(const PassArgs<double> &a, int CM, const SolveRows &r, cudaStream_t st) {
+    launch_solve_rows_impl<double>(a, CM, r, st);
 }
 
 }  // namespace tfs

@@ -68,6 +68,7 @@ struct PackArgs {
     int64_t row_base[kMaxModes + 1];
     int K, W, C, Cq, off_old, off_prev;
     const int32_t *S, *Q;
+    int prev_in_cur;  // the slices' cur regions hold the columns of Q (their final values)
     const int32_t *id_of[kMaxModes];  // slice row (rank) -> row id, per mode
 };
 
@@ -139,7 +140,6 @@ struct FoldArgs {
 };
 
 constexpr int kPassThreads = 128;
-constexpr int kCombineThreads = 512;
 
 int pick_cm(int C);  // smallest instantiated register width >= C (0 if none); C > 16
                      // takes the wide path (wide.cu) with CM = C rounded up to 4
@@ -187,6 +187,17 @@ void launch_sum_slot_groups(T *partials, int NB, const int32_t *groups, int n_gr
 template <class T>
 void launch_res_wide(const ResArgs<T> &a, int W, cudaStream_t st);
 
+// The rows of a mode as k_solve_rows takes them: rows of one slot, split rows of at most
+// kLightSlots slots (the first n_light of `split`) and the n_heavy split rows beyond.  A heavy
+// row's value v is summed by kSlotSums / NB threads (NB values per slot), each every
+// so-manieth slot; up to kLightSlots slots that is the plain order for every NB.
+constexpr int kLightSlots = 3;
+constexpr int kSlotSums = 512;
+struct SolveRows {
+    const SplitRow *single, *split;
+    int n_single, n_light, n_heavy;
+};
+
 // Launch plan of one cp.async mode pass: one block per SM, warps per block.
 struct PassPlan {
     int warps = 0, grid = 0;
@@ -197,11 +208,7 @@ PassPlan mode_pass_plan(int CM, int N, int n, bool first, int num_sms, int P);
 template <class T>
 void launch_mode_pass(const PassArgs<T> &a, int CM, const PassPlan &plan, cudaStream_t st);
 template <class T>
-void launch_combine(const PassArgs<T> &a, int CM, const SplitRow *rows, int n_rows,
-                    cudaStream_t st);
-template <class T>
-void launch_solve_rows(const PassArgs<T> &a, int CM, const SplitRow *rows, int n_rows,
-                       cudaStream_t st);
+void launch_solve_rows(const PassArgs<T> &a, int CM, const SolveRows &r, cudaStream_t st);
 template <class T>
 void launch_pack(const PackArgs<T> &a, cudaStream_t st);
 template <class T>
