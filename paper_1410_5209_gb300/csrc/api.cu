@@ -196,7 +196,7 @@ struct ModeLayout {
     Buf<int32_t> id_of;     // degree rank -> row id
     Buf<int32_t> groups;    // slot groups of split rows (first slot, count), wide subsets
     int n_groups = 0;
-    int n_light = 0;  // split rows of at most kLightSlots slots: the first of `split`
+    int n_light = 0, n_medium = 0;  // split rows by slot count (SolveRows), in that order
     std::vector<int64_t> deg_cum;  // host: entries of the first R rows in degree-rank order
     // per bin, the step units and entries of the bins before it (gather-plan regions)
     Buf<uint32_t> plan_base;  // [2 (P + 1)]
@@ -393,7 +393,7 @@ struct Impl : CtxBase {
         std::vector<int64_t> bin_ptr;
         std::vector<SplitRow> split, single;
         std::vector<int32_t> groups;  // slot groups of rows with many chunks (wide subsets)
-        int n_light = 0;  // split rows of at most kLightSlots slots: the first of `split`
+        int n_light = 0, n_medium = 0;  // split rows by slot count (SolveRows), in that order
         int64_t n_slots = 0;
         // gather-plan regions: step units (max(1, ceil(len / 32)) per item) and entries
         // of the bins before each bin, [P + 1] each
@@ -879,11 +879,13 @@ struct Impl : CtxBase {
             (q2 - q > 1 ? h.split : h.single).push_back(sr);
             q = q2;
         }
-        h.n_light = (int)(std::stable_partition(h.split.begin(), h.split.end(),
-                                                [](const SplitRow &r) {
-                                                    return r.n_slots <= kLightSlots;
-                                                }) -
-                          h.split.begin());
+        auto upto = [&](std::vector<SplitRow>::iterator from, int slots) {
+            return std::stable_partition(from, h.split.end(),
+                                         [=](const SplitRow &r) { return r.n_slots <= slots; });
+        };
+        const auto light = upto(h.split.begin(), kLightSlots), medium = upto(light, kHeavySlots);
+        h.n_light = (int)(light - h.split.begin());
+        h.n_medium = (int)(medium - light);
         for (const SplitRow &sr : h.split)
             if (sr.n_slots > kSlotGroup)
                 for (int g = 0; g < sr.n_slots; g += kSlotGroup) {
@@ -928,6 +930,7 @@ struct Impl : CtxBase {
         L.n_groups = (int)(h.groups.size() / 2);
         L.groups.alloc(std::max<size_t>(h.groups.size(), 2), st);
         L.n_light = h.n_light;
+        L.n_medium = h.n_medium;
         L.plan_base.alloc(h.plan_base.size(), st);
         L.plan_units = h.plan_units;
         stage.copy(L.groups.p, h.groups.data(), h.groups.size() * sizeof(int32_t), st);
@@ -1368,8 +1371,8 @@ struct Impl : CtxBase {
                         ++launches;
                     solved:
                         timed(TF_KIND_SOLVE, [&] {
-                            const SolveRows rows{L.single.p, L.split.p, L.n_single, L.n_light,
-                                                 L.n_split - L.n_light};
+                            const SolveRows rows{L.single.p, L.split.p,  L.n_single, L.n_light,
+                                                 L.n_medium, L.n_split - L.n_light - L.n_medium};
                             launch_solve_rows<T>(a, CM, rows, st);
                         });
                         ++launches;

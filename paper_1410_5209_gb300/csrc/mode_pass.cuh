@@ -781,18 +781,19 @@ __global__ void __launch_bounds__(pass_max_warps<T, CM>() * kWarp, 1)
 }
 
 // Row solves of a mode: (B + lambda I) a = c (Eq. 4) for every row, by the register Cholesky
-// of Section 3.1 with one lane per row, in one launch.
-//   Light rows (up to kLightSlots partial slots): a warp takes 32 of them.  It sums the
-//   rows' slots into shared memory with consecutive lanes on consecutive values, up to 24
-//   loads in flight per lane, and each lane then solves its row.
-//   Heavy rows: one block each; thread (g, v) adds value v of every G-th slot from g on
-//   (eight loads in flight), the G sums are added in order, one lane solves.
+// of Section 3.1 with one lane per row, in one launch.  A row with several slots is summed as
+// G = kSlotSums / NB sums of every G-th slot, added in order (plain order up to G slots).
+//   Heavy rows (more than kHeavySlots partial slots): one block each; a thread advances up to
+//   four of the G * NB sums together, 32 loads in flight.
+//   Medium rows: eight per block, two per warp, lanes over the values.
+//   Light rows (up to kLightSlots): 32 per warp, brought into shared memory with consecutive
+//   lanes on consecutive values; where the 32 slots lie together, as 16-byte cp.async.
 // Bound: latency, reading the slots (C = 10: 260 B a row) and the scattered columns of the
 // factor rows written (one 32-byte sector per value where K is large).  Before, one launch
 // solved the single-slot rows, each thread reading its row's slot at a stride of NB values,
 // and a second took 512 threads per split row: 44 + 55 us per mode of 1e5 rows (1e8 entries,
-// C = 10), now 70; 1,000 FP64 rows of two slots, C = 5: 127 us (a lone lane's FP64
-// instructions take the unit as long as a full warp's), now 25.
+// C = 10), now 61; 1,000 FP64 rows of two slots, C = 5: 127 us (a lone lane's FP64
+// instructions take the unit as long as a full warp's), now 19.
 // XS: the solve options of float contexts (refinement / FP64 fallback) are on; the plain
 // Cholesky otherwise, so that the default kernels carry none of their registers.
 template <class T, int CM, bool XS>
@@ -816,20 +817,31 @@ constexpr int kSolveThreads = 128;
 // Sum of a heavy row's slots at p into tot[NB]; red: G * NB values (both shared memory).
 template <class T, int NB>
 __device__ __forceinline__ void sum_slots(const T *p, int count, T *red, T *tot) {
-    constexpr int G = kSlotSums / NB, U = 8;
+    // a thread's sums (every kSolveThreads-th of the G * NB) advance together
+    constexpr int G = kSlotSums / NB, PT = (G * NB + kSolveThreads - 1) / kSolveThreads, U = 32 / PT;
     const int tid = threadIdx.x;
-    for (int t = tid; t < G * NB; t += kSolveThreads) {
-        const int g = t / NB, v = t - g * NB;
-        T s = T(0);
-        for (int k = g; k < count; k += U * G) {
-            T w[U];
+    T s[PT];
 #pragma unroll
-            for (int u = 0; u < U; ++u) w[u] = k + u * G < count ? p[(int64_t)(k + u * G) * NB + v] : T(0);
+    for (int i = 0; i < PT; ++i) s[i] = T(0);
+    for (int k = 0; k < count; k += U * G) {
+        T w[PT][U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) s += w[u];
+        for (int i = 0; i < PT; ++i) {
+            const int t = tid + i * kSolveThreads, g = t / NB, v = t - g * NB;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int slot = k + g + u * G;
+                w[i][u] = t < G * NB && slot < count ? p[(int64_t)slot * NB + v] : T(0);
+            }
         }
-        red[t] = s;
+#pragma unroll
+        for (int i = 0; i < PT; ++i)
+#pragma unroll
+            for (int u = 0; u < U; ++u) s[i] += w[i][u];
     }
+#pragma unroll
+    for (int i = 0; i < PT; ++i)
+        if (tid + i * kSolveThreads < G * NB) red[tid + i * kSolveThreads] = s[i];
     __syncthreads();
     for (int v = tid; v < NB; v += kSolveThreads) {
         T s = T(0);
@@ -839,60 +851,133 @@ __device__ __forceinline__ void sum_slots(const T *p, int count, T *red, T *tot)
     __syncthreads();
 }
 
-// A warp's 32 rows of sums (odd stride: lanes reading their rows do not conflict), or a
-// heavy row's group sums and total.
+// Sum of a medium row's slots at p into tot[NB] (shared memory) by one warp.
+template <class T, int NB>
+__device__ __forceinline__ void sum_slots_warp(const T *p, int count, T *tot, int lane) {
+    constexpr int G = kSlotSums / NB, VL = (NB + 31) / 32, U = VL > 2 ? 4 : 8;
+    T sum[VL];
+#pragma unroll
+    for (int i = 0; i < VL; ++i) sum[i] = T(0);
+    for (int g = 0; g < G && g < count; g += U) {
+        T s[VL][U];
+#pragma unroll
+        for (int i = 0; i < VL; ++i)
+#pragma unroll
+            for (int u = 0; u < U; ++u) s[i][u] = T(0);
+        for (int k = g; k < count; k += G) {
+            T w[VL][U];
+#pragma unroll
+            for (int i = 0; i < VL; ++i)
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    w[i][u] = g + u < G && k + u < count && lane + 32 * i < NB
+                                  ? p[(int64_t)(k + u) * NB + lane + 32 * i]
+                                  : T(0);
+#pragma unroll
+            for (int i = 0; i < VL; ++i)
+#pragma unroll
+                for (int u = 0; u < U; ++u) s[i][u] += w[i][u];
+        }
+#pragma unroll
+        for (int i = 0; i < VL; ++i)
+#pragma unroll
+            for (int u = 0; u < U; ++u) sum[i] += s[i][u];
+    }
+#pragma unroll
+    for (int i = 0; i < VL; ++i)
+        if (lane + 32 * i < NB) tot[lane + 32 * i] = sum[i];
+}
+
+// Values of a warp's 32 light rows in shared memory, and their row stride: flat where NB is
+// odd (lanes reading their rows do not conflict) or the conflicts are few, else one more.
+template <int NB>
+constexpr int solve_stride() {
+    return NB % 8 == 0 ? NB + 1 : NB;
+}
 template <class T, int CM>
 constexpr size_t solve_rows_smem() {
     constexpr int NB = CM * (CM + 1) / 2 + CM;
-    constexpr int light = kSolveThreads * (NB | 1), heavy = kSlotSums + NB;
-    return sizeof(T) * (size_t)(light > heavy ? light : heavy);
+    constexpr int light = kSolveThreads / 32 * ((32 * solve_stride<NB>() + 7) / 4 * 4);
+    constexpr int heavy = kSlotSums + NB, medium = kMediumRows * NB;
+    constexpr int most = light > heavy ? light : heavy;
+    return sizeof(T) * (size_t)(most > medium ? most : medium);
 }
 
 template <class T, int CM, bool XS>
 __global__ void __launch_bounds__(kSolveThreads) k_solve_rows(const PassArgs<T> a,
                                                               const SolveRows r) {
-    constexpr int NT = CM * (CM + 1) / 2, NB = NT + CM, NBP = NB | 1;
+    constexpr int NT = CM * (CM + 1) / 2, NB = NT + CM, NBP = solve_stride<NB>();
+    constexpr int V = 16 / (int)sizeof(T);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *sm = reinterpret_cast<T *>(smem_raw);
-    if ((int)blockIdx.x < r.n_heavy) {  // first, the longest
-        const SplitRow sr = r.split[r.n_light + blockIdx.x];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int blk = (int)blockIdx.x;
+    if (blk < r.n_heavy) {  // first, the longest
+        const SplitRow sr = r.split[r.n_light + r.n_medium + blk];
         T *tot = sm + kSlotSums;
         sum_slots<T, NB>(a.partials + (int64_t)sr.first_slot * NB, sr.n_slots, sm, tot);
         if (threadIdx.x == 0) solve_and_write<T, CM, XS>(a, sr, tot);
         return;
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int i = ((int)blockIdx.x - r.n_heavy) * kSolveThreads + (int)threadIdx.x;
+    blk -= r.n_heavy;
+    if (blk < (r.n_medium + kMediumRows - 1) / kMediumRows) {
+        const SplitRow *rows = r.split + r.n_light + blk * kMediumRows;
+        const int n = min(kMediumRows, r.n_medium - blk * kMediumRows);
+        for (int q = warp; q < n; q += kSolveThreads / 32)
+            sum_slots_warp<T, NB>(a.partials + (int64_t)rows[q].first_slot * NB, rows[q].n_slots,
+                                  sm + q * NB, lane);
+        __syncthreads();
+        if ((int)threadIdx.x < n)
+            solve_and_write<T, CM, XS>(a, rows[threadIdx.x], sm + threadIdx.x * NB);
+        return;
+    }
+    blk -= (r.n_medium + kMediumRows - 1) / kMediumRows;
+    const int i = blk * kSolveThreads + (int)threadIdx.x;
     SplitRow sr{};
     if (i < r.n_single)
         sr = r.single[i];
     else if (i < r.n_single + r.n_light)
         sr = r.split[i - r.n_single];
-    T *buf = sm + warp * 32 * NBP;
-    constexpr int U = 8;
-    const bool one = __all_sync(0xFFFFFFFFu, sr.n_slots <= 1);
-    for (int q0 = lane; q0 < 32 * NB; q0 += 32 * U) {
-        T s[U];
+    T *buf = sm + warp * ((32 * NBP + 7) / 4 * 4);
+    const int first0 = __shfl_sync(0xFFFFFFFFu, sr.first_slot, 0);
+    if (NBP == NB && __all_sync(0xFFFFFFFFu, sr.n_slots == 1 && sr.first_slot == first0 + lane)) {
+        // 32 slots in a row: copied as they lie, in whole vectors but for the ends
+        const int64_t e0 = (int64_t)first0 * NB;
+        const int skew = (int)(e0 % V), lead = skew ? V - skew : 0;
+        const T *src = a.partials + e0;
+        buf += skew;
+        const int nv = (32 * NB - lead) / V, tail = 32 * NB - lead - nv * V;
+        for (int q = lane; q < nv; q += 32) cp_async16(buf + lead + q * V, src + lead + q * V);
+        if (lane < lead) cp_async_small<sizeof(T)>(buf + lane, src + lane);
+        if (lane < tail) {
+            const int q = 32 * NB - tail + lane;
+            cp_async_small<sizeof(T)>(buf + q, src + q);
+        }
+        cp_async_commit();
+        cp_async_wait<0>();
+    } else {
+        constexpr int U = 8;
+        for (int q0 = lane; q0 < 32 * NB; q0 += 32 * U) {
+            T s[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int q = q0 + 32 * u, w = q / NB, v = q - w * NB;
-            const int first = __shfl_sync(0xFFFFFFFFu, sr.first_slot, w & 31);
-            const int n = __shfl_sync(0xFFFFFFFFu, sr.n_slots, w & 31);
-            const T *p = a.partials + (int64_t)first * NB + v;
-            const int ns = q < 32 * NB ? n : 0;
-            s[u] = ns > 0 ? p[0] : T(0);
-            if (!one) {
+            for (int u = 0; u < U; ++u) {
+                const int q = q0 + 32 * u, w = q / NB, v = q - w * NB;
+                const int first = __shfl_sync(0xFFFFFFFFu, sr.first_slot, w & 31);
+                const int n = __shfl_sync(0xFFFFFFFFu, sr.n_slots, w & 31);
+                const T *p = a.partials + (int64_t)first * NB + v;
+                const int ns = q < 32 * NB ? n : 0;
                 T t[kLightSlots];
 #pragma unroll
-                for (int k = 1; k < kLightSlots; ++k) t[k] = k < ns ? p[k * NB] : T(0);
+                for (int k = 0; k < kLightSlots; ++k) t[k] = k < ns ? p[k * NB] : T(0);
+                s[u] = t[0];
 #pragma unroll
                 for (int k = 1; k < kLightSlots; ++k) s[u] += t[k];
             }
-        }
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int q = q0 + 32 * u, w = q / NB, v = q - w * NB;
-            if (q < 32 * NB) buf[w * NBP + v] = s[u];
+            for (int u = 0; u < U; ++u) {
+                const int q = q0 + 32 * u, w = q / NB, v = q - w * NB;
+                if (q < 32 * NB) buf[w * NBP + v] = s[u];
+            }
         }
     }
     __syncwarp();
@@ -1038,9 +1123,17 @@ void launch_mode_pass_cm(const PassArgs<T> &a, const PassPlan &plan, cudaStream_
 }
 
 template <class T, int CM>
-void launch_solve_rows_cm(const PassArgs<T> &a, const SolveRows &r, cudaStream_t st) {
-    const int64_t blocks =
-        r.n_heavy + ((int64_t)r.n_single + r.n_light + kSolveThreads - 1) / kSolveThreads;
+void launch_solve_rows_cm(const PassArgs<T> &a, const SolveRows &rows, cudaStream_t st) {
+    SolveRows r = rows;
+    if (CM * (CM + 1) / 2 + CM < 32) {
+        // fewer values than lanes: a warp would leave lanes idle and walk the slots in more
+        // rounds than a block (C = 1, 2,000 medium rows: 10 against 8 us; C = 5 in FP64, 100
+        // rows: 18 against 14.5; the other way at C = 10, 1,500 rows: 60 against 70)
+        r.n_heavy += r.n_medium;
+        r.n_medium = 0;
+    }
+    const int64_t blocks = r.n_heavy + (r.n_medium + kMediumRows - 1) / kMediumRows +
+                           ((int64_t)r.n_single + r.n_light + kSolveThreads - 1) / kSolveThreads;
     if (blocks <= 0) return;
     const bool xs = sizeof(T) == 4 && (a.refine || a.cond_limit > 0.f);
     auto kern = xs ? k_solve_rows<T, CM, true> : k_solve_rows<T, CM, false>;

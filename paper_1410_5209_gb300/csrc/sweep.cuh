@@ -187,15 +187,17 @@ void launch_sum_slot_groups(T *partials, int NB, const int32_t *groups, int n_gr
 template <class T>
 void launch_res_wide(const ResArgs<T> &a, int W, cudaStream_t st);
 
-// The rows of a mode as k_solve_rows takes them: rows of one slot, split rows of at most
-// kLightSlots slots (the first n_light of `split`) and the n_heavy split rows beyond.  A heavy
-// row's value v is summed by kSlotSums / NB threads (NB values per slot), each every
-// so-manieth slot; up to kLightSlots slots that is the plain order for every NB.
+// The rows of a mode as k_solve_rows takes them: rows of one slot, and the split rows in the
+// order of `split`: n_light of at most kLightSlots slots, n_medium of at most kHeavySlots, and
+// n_heavy beyond.  (One warp would take a heavy row's slots in too many rounds of loads; a
+// block per medium row left 127 of 128 threads idle while one solved.)
 constexpr int kLightSlots = 3;
-constexpr int kSlotSums = 512;
+constexpr int kHeavySlots = 64;
+constexpr int kMediumRows = 8;   // per block
+constexpr int kSlotSums = 512;   // sums of slots formed side by side for one row
 struct SolveRows {
     const SplitRow *single, *split;
-    int n_single, n_light, n_heavy;
+    int n_single, n_light, n_medium, n_heavy;
 };
 
 // Launch plan of one cp.async mode pass: one block per SM, warps per block.
