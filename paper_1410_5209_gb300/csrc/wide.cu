@@ -25,13 +25,6 @@ constexpr int kWideThreads = 256;
 constexpr int kWideTile = 32;        // entries per tile
 constexpr int kSolveWarps = 4;        // rows per solve block
 
-template <class T>
-__device__ __forceinline__ T wsum(T v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-    return v;
-}
-
 // 16-byte vector of slice values (4 floats or 2 doubles).
 template <class T>
 struct Vec16;
@@ -686,13 +679,18 @@ __global__ void __launch_bounds__(256) k_sum_slot_groups(T *partials, int NB,
     }
 }
 
-// Residual of copy n against the cur region of the slices: one warp per bin, lanes
-// over columns; what = 0 sums r^2 per block (fixed order), 1 scatters r to canonical
-// order, 2 writes r back to the copy.
+// Residual of copy n against the cur region of the slices: one warp per bin, eight entries at
+// a time (lane 4 g + t takes entries t and t + 4 and the columns of 16-byte vectors g, g + 8,
+// ... of their rows; regions start at multiples of CM, a multiple of four); what = 0 sums r^2
+// per block (fixed order), 1 scatters r to canonical order, 2 writes r back to the copy.
+// Bound: the gathers' latency.  The loss of 1e7 entries at C = 50: 1.72 ms one entry at a time
+// with lanes over single columns, 0.77 ms now.
 template <class T>
 __global__ void __launch_bounds__(kWideThreads) k_res_wide(const ResArgs<T> a, int W) {
+    using V = typename Vec16<T>::type;
+    constexpr int VW = Vec16<T>::n;
     __shared__ double wsum_d[kWideThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     const int bin = blockIdx.x * (kWideThreads / 32) + warp;
     const int no = a.N - 1;
     double acc = 0.0;
@@ -700,22 +698,49 @@ __global__ void __launch_bounds__(kWideThreads) k_res_wide(const ResArgs<T> a, i
         for (int64_t it = a.bin_ptr[bin]; it < a.bin_ptr[bin + 1]; ++it) {
             const tf_item item = a.items[it];
             const T *own = a.Zn + (int64_t)a.rank_n[item.row] * W;
-            for (int64_t j = item.begin; j < item.begin + item.len; ++j) {
-                T p = T(0);
-                for (int c = lane; c < a.Cq; c += 32) {
-                    T q = own[c];
-                    for (int t = 0; t < no; ++t) q *= a.Zo[t][(int64_t)a.oidx[t][j] * W + c];
-                    p += q;
+            const int64_t end = item.begin + item.len;
+            for (int64_t j0 = item.begin; j0 < end; j0 += 8) {
+                T p[2] = {T(0), T(0)}, rv[2] = {T(0), T(0)};
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+                    if (j0 + t + 4 * e < end) rv[e] = a.res[j0 + t + 4 * e];
+                for (int c = VW * g; c < a.Cq; c += 8 * VW) {
+                    T o[VW];
+                    Vec16<T>::unpack(*reinterpret_cast<const V *>(own + c), o);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int64_t j = j0 + t + 4 * e;
+                        if (j >= end) continue;
+                        T q[VW];
+#pragma unroll
+                        for (int u = 0; u < VW; ++u) q[u] = o[u];
+                        for (int m = 0; m < no; ++m) {
+                            T x[VW];
+                            Vec16<T>::unpack(*reinterpret_cast<const V *>(
+                                                 a.Zo[m] + (int64_t)a.oidx[m][j] * W + c),
+                                             x);
+#pragma unroll
+                            for (int u = 0; u < VW; ++u) q[u] *= x[u];
+                        }
+#pragma unroll
+                        for (int u = 0; u < VW; ++u)
+                            if (c + u < a.Cq) p[e] += q[u];
+                    }
                 }
-                p = wsum(p);
-                const T r = a.res[j] - p;
-                if (lane == 0) {
-                    if (a.what == 0)
-                        acc += (double)r * (double)r;
-                    else if (a.what == 1)
-                        a.out[a.perm[j]] = r;
-                    else
-                        a.res[j] = r;
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+#pragma unroll
+                    for (int o = 4; o < 32; o <<= 1) p[e] += __shfl_xor_sync(0xFFFFFFFFu, p[e], o);
+                    const int64_t j = j0 + t + 4 * e;
+                    if (g == 0 && j < end) {
+                        const T r = rv[e] - p[e];
+                        if (a.what == 0)
+                            acc += (double)r * (double)r;
+                        else if (a.what == 1)
+                            a.out[a.perm[j]] = r;
+                        else
+                            a.res[j] = r;
+                    }
                 }
             }
         }
