@@ -242,6 +242,7 @@ struct Impl : CtxBase {
     ModeLayout mode[kMaxModes];
     Buf<T> partials;
     Buf<int32_t> d_order, d_Q;
+    Buf<uint32_t> wide_mx;  // largest current column values of wide sweeps (wide_max)
     Buf<DeviceStatus> stat;
     Buf<unsigned long long> ticket;  // bin counter of the mode passes
     unsigned long long ticket_base = 0;
@@ -304,7 +305,8 @@ struct Impl : CtxBase {
     // Every device buffer of the context (tf_set_stream moves their frees to the new stream).
     template <class F>
     void each_buf(F f) {
-        f(x), f(partials), f(d_order), f(d_Q), f(stat), f(ticket), f(red), f(d_dims);
+        f(x), f(partials), f(d_order), f(d_Q), f(stat), f(ticket), f(red), f(d_dims),
+            f(wide_mx);
         f(f_other), f(f_x), f(f_out), f(f_part), f(f_fac), f(f_rpart), f(f_meta), f(p_coords),
             f(p_out);
         for (int n = 0; n < kMaxModes; ++n) {
@@ -1120,6 +1122,12 @@ struct Impl : CtxBase {
         return d;
     }
 
+    // Largest |current column value| of mode l in split s: 0 after the pack, t + 1 after inner
+    // iteration t (PassArgs::mx).
+    uint32_t *wide_max(int s, int when, int l, int T_in) {
+        return wide_mx.p + ((size_t)s * (T_in + 1) + when) * N + l;
+    }
+
     // ------------------------------------------------------------ the sweep
     void sweep(int C, double lambda, int T_in, const int32_t *order, uint32_t flags) {
         if (C < 1 || C > K) throw ApiError{TF_EINVAL, "C must be in 1..K"};
@@ -1199,10 +1207,23 @@ struct Impl : CtxBase {
                 }
         last_path = 0;
         const int nsplit = (K + C - 1) / C;
+        // Wide subsets of float three-way tensors up to C = 63, without solve options: the
+        // warp-wide pass with register operands (mma_pass.cu), unless path 1 or 2 or the
+        // single-TF32 form asks for another.  Against the block-wide passes: 5e6 entries at
+        // C = 20 0.28 against 0.75 ms a pass, 1e7 at C = 50 1.83 against 2.60 ms.  Errors of
+        // the factors against 64 bits over nine drawn tensors: C <= 31 0.9 to 1.1 times the
+        // SIMT pass's (4.6e-7 to 1.6e-6), C >= 32 a third of the tcgen05 pass's.
+        const bool wide_mma = sizeof(T) == 4 && wide && path != 1 && path != 2 && precision != 1 &&
+                              pass_mma_supported(N, C, CM) &&
+                              solve_mid_supported(C, solve_refine || solve_cond > 0.f);
+        if (wide_mma) wide_mx.ensure((size_t)nsplit * (T_in + 1) * N, st);
         // every launch of the splits (pack, mode passes, solves) and the copy of the last
         // split's columns into Q; returns |Q|
         auto run_splits = [&]() {
             int cq = Cq;
+            if (wide_mma)
+                TFS_CUDA(cudaMemsetAsync(wide_mx.p, 0, (size_t)nsplit * (T_in + 1) * N * sizeof(uint32_t),
+                                         st));
             const int32_t *Qp = d_Q.p;
             for (int s = 0; s < nsplit; ++s) {
                 const int Cs = (s == nsplit - 1) ? K - s * C : C;
@@ -1225,6 +1246,7 @@ struct Impl : CtxBase {
                 pk.S = Sp;
                 pk.Q = Qp;
                 pk.prev_in_cur = s > 0;
+                pk.mx = wide_mma ? wide_max(s, 0, 0, T_in) : nullptr;
                 timed(TF_KIND_PACK, [&] { launch_pack<T>(pk, st); });
                 ++launches;
                 if (bf16_rows) {
@@ -1269,20 +1291,59 @@ struct Impl : CtxBase {
                         a.ticket = ticket.p;
                         a.ticket_base = ticket_base;
                         if (wide) {
-                            // float: the Gram on the tensor cores for 64- and 128-wide tiles
-                            // (C >= 32: faster than the SIMT Gram at 1e8 entries) or when
-                            // requested (path 2, precision 1); SIMT for 32-wide tiles and
-                            // on path 1
+                            // the block-wide pass: its Gram on the tensor cores for 64- and
+                            // 128-wide tiles (C >= 32: faster than SIMT FMAs at 1e8 entries)
+                            // or when requested (path 2, precision 1); SIMT for 32-wide tiles
+                            // and on path 1
                             const bool tc = sizeof(T) == 4 && path != 1 &&
                                             (path == 2 || precision == 1 ||
                                              wide_split_width(Cs, CM) >= 64);
+                            if (wide_mma) {
+                                if constexpr (sizeof(T) == 4) {
+                                    const PassPlan plan = pass_mma_plan(Cs, CM, pass_sms(), L.P);
+                                    for (int u = 0; u < 2; ++u) {
+                                        const int l = L.omode[u];
+                                        a.mx[u] = wide_max(s, l < n ? t + 1 : t, l, T_in);
+                                    }
+                                    a.mx_out = wide_max(s, t + 1, n, T_in);
+                                    a.gate = 1;
+                                    a.gate_tickets = (unsigned long long)L.P +
+                                                     (unsigned long long)plan.grid * plan.warps;
+                                    timed(TF_KIND_MODE_PASS,
+                                          [&] { launch_pass_mma(a, CM, W, plan.grid, st); });
+                                    ticket_base += a.gate_tickets;
+                                    a.ticket_base = ticket_base;
+                                    a.gate = 2;
+                                    last_path |= 4;
+                                    ++launches;
+                                }
+                            }
                             const int wgrid = pass_wide_grid<T>(pass_sms(), L.P, Cs, CM, tc, t == 0);
                             // every block takes one ticket past the last bin
-                            ticket_base += (unsigned long long)L.P + (unsigned long long)wgrid;
+                            a.gate_tickets = (unsigned long long)L.P + (unsigned long long)wgrid;
+                            ticket_base += a.gate_tickets;
                             timed(TF_KIND_MODE_PASS,
                                   [&] { launch_pass_wide<T>(a, CM, W, wgrid, tc, precision != 1, st); });
                             last_path |= tc ? 4 : 1;
                             ++launches;
+                            if constexpr (sizeof(T) == 4) {
+                                if (solve_mid_supported(Cs, solve_refine || solve_cond > 0.f)) {
+                                    if (L.n_groups > 0) {
+                                        timed(TF_KIND_COMBINE, [&] {
+                                            launch_sum_slot_groups<T>(partials.p,
+                                                                      partial_stride(CM),
+                                                                      L.groups.p, L.n_groups, st);
+                                        });
+                                        ++launches;
+                                    }
+                                    timed(TF_KIND_SOLVE, [&] {
+                                        launch_solve_mid(a, L.split.p, L.n_split, L.single.p,
+                                                         L.n_single, CM, W, st);
+                                    });
+                                    ++launches;
+                                    continue;
+                                }
+                            }
                             if (L.n_single > 0) {
                                 timed(TF_KIND_SOLVE, [&] {
                                     launch_solve_wide<T>(a, L.single.p, L.n_single, CM, W, st);
@@ -1402,7 +1463,8 @@ struct Impl : CtxBase {
             gk.C = C, gk.T_in = T_in, gk.CM = CM, gk.Cq = Cq, gk.path = path;
             gk.precision = precision, gk.use_tma = use_tma, gk.flags = flags;
             gk.refine = solve_refine, gk.cond = solve_cond;
-            gk.lambda = lambda, gk.layout_gen = layout_gen, gk.partials = partials.p;
+            gk.lambda = lambda, gk.layout_gen = layout_gen, gk.partials = partials.p,
+            gk.wide_mx = wide_mx.p;
             for (int l = 0; l < N; ++l) {
                 gk.Z[l] = Z[l].p;
                 gk.Zb[l] = Zb[l].p;
@@ -1429,14 +1491,15 @@ struct Impl : CtxBase {
         uint32_t flags;
         double lambda;
         int64_t layout_gen;
-        const void *partials;
+        const void *partials, *wide_mx;
         const void *Z[kMaxModes];
         const void *Zb[kMaxModes];
         bool operator==(const GraphKey &o) const {
             if (C != o.C || T_in != o.T_in || CM != o.CM || Cq != o.Cq || path != o.path ||
                 precision != o.precision || refine != o.refine || cond != o.cond ||
                 use_tma != o.use_tma || flags != o.flags ||
-                lambda != o.lambda || layout_gen != o.layout_gen || partials != o.partials)
+                lambda != o.lambda || layout_gen != o.layout_gen || partials != o.partials ||
+                wide_mx != o.wide_mx)
                 return false;
             for (int l = 0; l < kMaxModes; ++l)
                 if (Z[l] != o.Z[l] || Zb[l] != o.Zb[l]) return false;

@@ -56,9 +56,17 @@ __global__ void __launch_bounds__(kPackThreads) k_pack(const PackArgs<T> a) {
     const int CM = a.off_prev, rows = kPackThreads / CM;
     const int w = (int)threadIdx.x / CM, c = (int)threadIdx.x - w * CM;
     const int64_t r = (int64_t)blockIdx.x * rows + w;
-    if (w >= rows || r >= a.row_base[a.N]) return;
+    const bool live = w < rows && r < a.row_base[a.N];
+    if (!a.mx && !live) return;
     int l = 0;
-    while (r >= a.row_base[l + 1]) ++l;
+    while (live && r >= a.row_base[l + 1]) ++l;
+    if (a.mx) {  // wide float passes: largest value per mode (mostly one mode per warp)
+        const float v =
+            live && c < a.C ? (float)a.A[l][(int64_t)a.id_of[l][r - a.row_base[l]] * a.K + a.S[c]] : 0.f;
+        for (int m = 0; m < a.N; ++m)
+            if (__any_sync(0xFFFFFFFFu, live && l == m)) record_max(a.mx + m, l == m ? v : 0.f);
+    }
+    if (!live) return;
     const int64_t i = r - a.row_base[l];  // slice row (rank)
     const T *Ar = a.A[l] + (int64_t)a.id_of[l][i] * a.K;
     T *z = a.Z[l] + i * a.W;

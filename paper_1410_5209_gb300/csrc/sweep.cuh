@@ -58,7 +58,35 @@ struct PassArgs {
     int refine;
     float cond_limit;
     double *loss_out;  // lean loss pass: per-item (slot) sums of r^2 (other passes: unused)
+    // wide passes of float three-way tensors: bits of the largest |current column value| of the
+    // two other modes (mx), where to record this mode's new one (mx_out; null: nowhere), and
+    // which of two launches of a pass this is (gate: 0 the only one, 1 the one that takes
+    // products in the range of wide_gate, 2 the one that takes the others)
+    const uint32_t *mx[2];
+    uint32_t *mx_out;
+    int gate;
+    unsigned long long gate_tickets;  // tickets the launch takes in all when it runs
 };
+
+#ifdef __CUDACC__
+// Whether this launch of a gated wide pass is the one that works; the one that does not takes
+// its tickets at once (block 0), which keeps the counter where the host expects it.
+template <class T>
+__device__ __forceinline__ bool wide_gate(const PassArgs<T> &a) {
+    if (a.gate == 0) return true;
+    const float m0 = __uint_as_float(*a.mx[0]), m1 = __uint_as_float(*a.mx[1]);
+    const double p = (double)m0 * (double)m1;
+    const bool fits = p == 0.0 || (p >= 0x1p-80 && p < 0x1p60);  // NaN: no
+    if (fits == (a.gate == 1)) return true;
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(a.ticket, a.gate_tickets);
+    return false;
+}
+// Records |v| (bits, one value per lane of the whole warp) as a maximum.
+__device__ __forceinline__ void record_max(uint32_t *slot, float v) {
+    const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(v) & 0x7FFFFFFFu);
+    if ((threadIdx.x & 31) == 0 && m > *(volatile uint32_t *)slot) atomicMax(slot, m);
+}
+#endif
 
 template <class T>
 struct PackArgs {
@@ -69,6 +97,7 @@ struct PackArgs {
     int K, W, C, Cq, off_old, off_prev;
     const int32_t *S, *Q;
     int prev_in_cur;  // the slices' cur regions hold the columns of Q (their final values)
+    uint32_t *mx;     // [N] bits of the largest |cur| value per mode (PassArgs::mx), or null
     const int32_t *id_of[kMaxModes];  // slice row (rank) -> row id, per mode
 };
 
@@ -184,6 +213,11 @@ constexpr int kSlotGroup = 64;
 template <class T>
 void launch_sum_slot_groups(T *partials, int NB, const int32_t *groups, int n_groups,
                             cudaStream_t st);
+// One-warp-per-row register solves for C <= 63 (mid_solve.cu): float contexts without
+// refinement or FP64 fallback; the slots of split rows in groups as above.
+bool solve_mid_supported(int C, bool options);
+void launch_solve_mid(const PassArgs<float> &a, const SplitRow *split, int n_split,
+                      const SplitRow *single, int n_single, int CM, int W, cudaStream_t st);
 template <class T>
 void launch_res_wide(const ResArgs<T> &a, int W, cudaStream_t st);
 
@@ -205,6 +239,11 @@ struct PassPlan {
     int warps = 0, grid = 0;
     size_t smem = 0;
 };
+// Wide pass of float three-way tensors for C <= 63 (mma_pass.cu); the plan has no dynamic
+// shared memory to hand on.
+bool pass_mma_supported(int N, int C, int CM);
+PassPlan pass_mma_plan(int C, int CM, int num_sms, int P);
+void launch_pass_mma(const PassArgs<float> &a, int CM, int W, int grid, cudaStream_t st);
 template <class T>
 PassPlan mode_pass_plan(int CM, int N, int n, bool first, int num_sms, int P);
 template <class T>

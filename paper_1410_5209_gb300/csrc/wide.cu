@@ -123,6 +123,7 @@ template <class T, int CW, bool FIRST>
 __global__ void __launch_bounds__(kWideThreads) k_pass_wide(const PassArgs<T> a, int CM, int W) {
     constexpr int R = CW / 16;       // register tile edge
     constexpr int HS = CW + 4;       // H row stride (elements)
+    if (!wide_gate(a)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *H = reinterpret_cast<T *>(smem_raw);           // [kWideTile][HS]
     T *own = H + kWideTile * HS;                       // prev | old of the own row (2 CM)
@@ -323,6 +324,7 @@ __global__ void __launch_bounds__(kWideThreads, CW >= 64 ? 3 : 1)
     k_pass_wide_tc(const PassArgs<float> a, int CM, int W) {
     using T = float;
     constexpr int kTcCols = CW;  // tensor-memory columns: the accumulator is 128 x CW fp32
+    if (!wide_gate(a)) return;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // kTcStages operand stages (hi and lo copies each)
     unsigned char *stage0 = smem_raw;
@@ -746,6 +748,7 @@ __global__ void __launch_bounds__(kWideThreads) k_res_wide(const ResArgs<T> a, i
         }
     }
     if (a.what != 0) return;
+    acc = warp_sum_d(acc);
     if (lane == 0) wsum_d[warp] = acc;
     __syncthreads();
     if (threadIdx.x == 0) {
