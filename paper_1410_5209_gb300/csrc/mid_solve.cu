@@ -5,7 +5,7 @@
 // memory as 16-byte broadcasts.
 //
 // Bound: the chain of C columns (pivot, broadcast, update: about 170 cycles each) with 12 warps
-// per SM in flight, against 1,300 packed FMAs and 520 broadcasts a row at C = 63.  The form it
+// per SM in flight, and issue: 1,300 packed FMAs and 520 broadcasts a row at C = 63.  The form it
 // replaces (k_solve_wide, wide.cu, still used for wider subsets, FP64 and the solve options)
 // walks a packed triangle in shared memory, two loads per multiply-add and a warp reduction
 // per column: 50,021 rows at C = 50 took it 1.06 ms (0.64 here), 30,011 at C = 20 0.26 (0.074).
@@ -42,38 +42,49 @@ __device__ __forceinline__ u64 mid_fma(u64 l, u64 m, u64 a) {
     return d;
 }
 
+// KM: columns held (C + 1 <= KM, a multiple of eight): 24 or 32 with one row per lane, up to 64
+// with two.  The work grows with KM^2 and the unrolled code with it.
+__host__ __device__ constexpr int mid_rows(int KM) { return KM <= 32 ? 1 : 2; }
 // Row stride of the factor in shared memory: 16-byte stores one row per lane do not conflict.
-__host__ __device__ constexpr int mid_ld(int R) { return 32 * R + 4; }
+__host__ __device__ constexpr int mid_ld(int KM) { return 32 * mid_rows(KM) + 4; }
 // Per warp: the factor's rows (the packed system before), and two column buffers.
-__host__ __device__ constexpr int mid_warp_floats(int R) { return 32 * R * mid_ld(R) + 64 * R; }
+__host__ __device__ constexpr int mid_warp_floats(int KM) {
+    return 32 * mid_rows(KM) * mid_ld(KM) + 64 * mid_rows(KM);
+}
 
 // Solves the system whose packed lower triangle is P[ntc] followed by the right-hand side [C]
 // (shared memory, overwritten).  x0 / x1: the solution's values lane and lane + 32.
-template <int R>
+template <int KM>
 __device__ __forceinline__ bool mid_solve(float *P, float *col, int C, float lam, int lane,
                                           float &x0, float &x1) {
-    constexpr int LD = mid_ld(R);
+    constexpr int R = mid_rows(KM), LD = mid_ld(KM);
+    constexpr int K0 = KM < 32 ? KM : 32;
     const int ntc = C * (C + 1) / 2;
-    u64 a0[16], a1[R == 2 ? 32 : 1];  // rows lane (columns 0-31) and lane + 32 (0-63), in pairs
-    auto value = [&](int i, int k) -> float {
-        if (i < C) return k <= i ? P[i * (i + 1) / 2 + k] + (k == i ? lam : 0.f) : 0.f;
-        return i == C && k < C ? P[ntc + k] : 0.f;
-    };
+    for (int i = lane; i < C; i += 32) P[i * (i + 1) / 2 + i] += lam;
+    __syncwarp();
+    // Rows lane (columns 0 .. 31) and lane + 32 (0 .. KM - 1), in pairs.  What is read past a
+    // row's end (the next rows, the rest of the buffer) ends up above the diagonal, in columns
+    // from C on or in rows past C, none of which reach the factor or the solution.
+    u64 a0[K0 / 2], a1[R == 2 ? KM / 2 : 1];
+    {
+        const float *p0 = P + (lane < C ? lane * (lane + 1) / 2 : ntc);
 #pragma unroll
-    for (int p = 0; p < 16; ++p) a0[p] = mid_pack(value(lane, 2 * p), value(lane, 2 * p + 1));
-    if constexpr (R == 2) {
+        for (int p = 0; p < K0 / 2; ++p) a0[p] = mid_pack(p0[2 * p], p0[2 * p + 1]);
+        if constexpr (R == 2) {
+            const int i = lane + 32;
+            const float *p1 = P + (i < C ? i * (i + 1) / 2 : ntc);
 #pragma unroll
-        for (int p = 0; p < 32; ++p)
-            a1[p] = mid_pack(value(lane + 32, 2 * p), value(lane + 32, 2 * p + 1));
+            for (int p = 0; p < KM / 2; ++p) a1[p] = mid_pack(p1[2 * p], p1[2 * p + 1]);
+        }
     }
     __syncwarp();
     bool ok = true;
     float inv0 = 1.f, inv1 = 1.f;  // inverse pivots of the lane's rows
 #pragma unroll
-    for (int j = 0; j < 32 * R; ++j) {
+    for (int j = 0; j < KM - 1; ++j) {
         if (j < C) {
             float *c = col + (j & 1) * 32 * R;
-            const float mine = j < 32 ? mid_get(a0[j < 32 ? j / 2 : 0], j & 1)
+            const float mine = j < 32 ? mid_get(a0[j < K0 ? j / 2 : 0], j & 1)
                                       : mid_get(a1[R == 2 ? j / 2 : 0], j & 1);
             float d = __shfl_sync(0xFFFFFFFFu, mine, j & 31);
             ok = ok && (d > 0.f);
@@ -84,7 +95,7 @@ __device__ __forceinline__ bool mid_solve(float *P, float *col, int C, float lam
             if (j < 32) {
                 l0 = lane == j ? d * inv : mine * inv;
                 if (lane == j) inv0 = inv;
-                a0[j < 32 ? j / 2 : 0] = mid_set(a0[j < 32 ? j / 2 : 0], j & 1, l0);
+                a0[j < K0 ? j / 2 : 0] = mid_set(a0[j < K0 ? j / 2 : 0], j & 1, l0);
                 c[lane] = l0;
             }
             if constexpr (R == 2) {
@@ -97,7 +108,7 @@ __device__ __forceinline__ bool mid_solve(float *P, float *col, int C, float lam
             __syncwarp();
             const u64 n0 = mid_pack(-l0, -l0), n1 = mid_pack(-l1, -l1);
 #pragma unroll
-            for (int q = 0; q < 8 * R; ++q) {
+            for (int q = 0; q < KM / 4; ++q) {
                 if (4 * q + 3 > j) {
                     const float4 v = *reinterpret_cast<const float4 *>(c + 4 * q);
                     const float w[4] = {v.x, v.y, v.z, v.w};
@@ -107,7 +118,7 @@ __device__ __forceinline__ bool mid_solve(float *P, float *col, int C, float lam
                         if (k + 1 <= j) continue;
                         // column j itself is finished: its half of the pair takes no update
                         const u64 l = mid_pack(k > j ? w[2 * h] : 0.f, w[2 * h + 1]);
-                        if (j < 32 && k < 32) a0[k < 32 ? k / 2 : 0] = mid_fma(l, n0, a0[k < 32 ? k / 2 : 0]);
+                        if (j < 32 && k < 32) a0[k < K0 ? k / 2 : 0] = mid_fma(l, n0, a0[k < K0 ? k / 2 : 0]);
                         if constexpr (R == 2) a1[k / 2] = mid_fma(l, n1, a1[k / 2]);
                     }
                 }
@@ -117,13 +128,13 @@ __device__ __forceinline__ bool mid_solve(float *P, float *col, int C, float lam
     // the factor's rows, L^-1 c as row C
     float *L = P;
 #pragma unroll
-    for (int p = 0; p < 8; ++p)
+    for (int p = 0; p < K0 / 4; ++p)
         *reinterpret_cast<float4 *>(L + lane * LD + 4 * p) =
             make_float4(mid_get(a0[2 * p], 0), mid_get(a0[2 * p], 1), mid_get(a0[2 * p + 1], 0),
                         mid_get(a0[2 * p + 1], 1));
     if constexpr (R == 2) {
 #pragma unroll
-        for (int p = 0; p < 16; ++p)
+        for (int p = 0; p < KM / 4; ++p)
             *reinterpret_cast<float4 *>(L + (lane + 32) * LD + 4 * p) =
                 make_float4(mid_get(a1[2 * p], 0), mid_get(a1[2 * p], 1), mid_get(a1[2 * p + 1], 0),
                             mid_get(a1[2 * p + 1], 1));
@@ -149,16 +160,17 @@ __device__ __forceinline__ bool mid_solve(float *P, float *col, int C, float lam
     return ok;
 }
 
-template <int R>
+template <int KM>
 __global__ void __launch_bounds__(kMidThreads) k_solve_mid(const PassArgs<float> a,
                                                            const SplitRow *split, int n_split,
                                                            const SplitRow *single, int n_single,
                                                            int CM, int W) {
+    constexpr int R = mid_rows(KM);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, C = a.C;
     const int NT = CM * (CM + 1) / 2, NB = NT + CM, ntc = C * (C + 1) / 2;
-    float *P = reinterpret_cast<float *>(smem_raw) + warp * mid_warp_floats(R);
-    float *col = P + 32 * R * mid_ld(R);
+    float *P = reinterpret_cast<float *>(smem_raw) + warp * mid_warp_floats(KM);
+    float *col = P + 32 * R * mid_ld(KM);
     SplitRow sr;
     if ((int)blockIdx.x < n_split) {
         sr = split[blockIdx.x];
@@ -204,7 +216,7 @@ __global__ void __launch_bounds__(kMidThreads) k_solve_mid(const PassArgs<float>
     }
     const float lam = a.weighted ? a.lambda * (float)sr.len : a.lambda;
     float x0, x1;
-    const bool ok = mid_solve<R>(P, col, C, lam, lane, x0, x1);
+    const bool ok = mid_solve<KM>(P, col, C, lam, lane, x0, x1);
     float *z = a.Zn + (int64_t)a.rank_n[sr.row] * W;
     float *Ar = a.A_n + (int64_t)sr.row * a.K;
     const bool in0 = lane < C, in1 = R == 2 && lane + 32 < C;
@@ -228,13 +240,13 @@ __global__ void __launch_bounds__(kMidThreads) k_solve_mid(const PassArgs<float>
     }
 }
 
-template <int R>
-void launch_solve_mid_r(const PassArgs<float> &a, const SplitRow *split, int n_split,
-                        const SplitRow *single, int n_single, int CM, int W, cudaStream_t st) {
+template <int KM>
+void launch_solve_mid_km(const PassArgs<float> &a, const SplitRow *split, int n_split,
+                         const SplitRow *single, int n_single, int CM, int W, cudaStream_t st) {
     constexpr int wpb = kMidThreads / 32;
-    const size_t smem = sizeof(float) * wpb * (size_t)mid_warp_floats(R);
-    TFS_CUDA(raise_smem_limit((const void *)k_solve_mid<R>, (int)smem));
-    k_solve_mid<R><<<n_split + (n_single + wpb - 1) / wpb, kMidThreads, smem, st>>>(
+    const size_t smem = sizeof(float) * wpb * (size_t)mid_warp_floats(KM);
+    TFS_CUDA(raise_smem_limit((const void *)k_solve_mid<KM>, (int)smem));
+    k_solve_mid<KM><<<n_split + (n_single + wpb - 1) / wpb, kMidThreads, smem, st>>>(
         a, split, n_split, single, n_single, CM, W);
     TFS_CUDA(cudaGetLastError());
 }
@@ -246,10 +258,13 @@ bool solve_mid_supported(int C, bool options) { return C <= 63 && !options; }
 void launch_solve_mid(const PassArgs<float> &a, const SplitRow *split, int n_split,
                       const SplitRow *single, int n_single, int CM, int W, cudaStream_t st) {
     if (n_split + n_single <= 0) return;
-    if (a.C <= 31)
-        launch_solve_mid_r<1>(a, split, n_split, single, n_single, CM, W, st);
-    else
-        launch_solve_mid_r<2>(a, split, n_split, single, n_single, CM, W, st);
+    auto launch = a.C < 24   ? launch_solve_mid_km<24>
+                  : a.C < 32 ? launch_solve_mid_km<32>
+                  : a.C < 40 ? launch_solve_mid_km<40>
+                  : a.C < 48 ? launch_solve_mid_km<48>
+                  : a.C < 56 ? launch_solve_mid_km<56>
+                             : launch_solve_mid_km<64>;
+    launch(a, split, n_split, single, n_single, CM, W, st);
 }
 
 }  // namespace tfs

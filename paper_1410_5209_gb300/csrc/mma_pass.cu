@@ -38,6 +38,16 @@ __device__ __forceinline__ float tf32_round(float x) {
     asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
     return __uint_as_float(r);
 }
+// d = A B: the first product of a chain (no zeros to move into place)
+__device__ __forceinline__ void mma8z(float (&d)[4], float a0, float a1, float a2, float a3, float b0,
+                                      float b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+        "{%8, %9}, {%10, %10, %10, %10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(__float_as_uint(a0)), "r"(__float_as_uint(a1)), "r"(__float_as_uint(a2)),
+          "r"(__float_as_uint(a3)), "r"(__float_as_uint(b0)), "r"(__float_as_uint(b1)), "f"(0.f));
+}
 // d += A B: A 16 x 8, B 8 x 8, TF32
 __device__ __forceinline__ void mma8(float (&d)[4], float a0, float a1, float a2, float a3, float b0,
                                      float b1) {
@@ -54,11 +64,24 @@ __device__ __forceinline__ u64 add2(u64 a, float lo, float hi) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
-__device__ __forceinline__ float4 ld4(const float *p, bool ok) {
-    return ok ? *reinterpret_cast<const float4 *>(p) : make_float4(0.f, 0.f, 0.f, 0.f);
+__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
+    u64 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
 }
-__device__ __forceinline__ void unpack4(const float4 &v, float (&x)[4]) {
-    x[0] = v.x, x[1] = v.y, x[2] = v.z, x[3] = v.w;
+__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
+    u64 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ void halves(u64 v, float &x, float &y) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
+// four columns of a row as two pairs, or zeros
+__device__ __forceinline__ void ld4(const float *p, bool ok, u64 (&v)[2]) {
+    ulonglong2 q = make_ulonglong2(0ull, 0ull);
+    if (ok) q = *reinterpret_cast<const ulonglong2 *>(p);
+    v[0] = q.x, v[1] = q.y;
 }
 
 // bfloat16 pair of (x, y), x in the lower half, and what it leaves of them
@@ -77,6 +100,15 @@ __device__ __forceinline__ void mma16(float (&d)[4], uint32_t a0, uint32_t a1, u
         "{%8, %9}, {%0, %1, %2, %3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ void mma16z(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
+                                       uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+        "{%8, %9}, {%10, %10, %10, %10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
 }
 
 // Entries per step: 16 (two halves of 8) for one chunk, 8 for two.
@@ -100,7 +132,7 @@ __global__ void __launch_bounds__(mma_warps(CH) * kWarp, 1)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint16_t *place = reinterpret_cast<uint16_t *>(smem_raw);  // [NV][32]: value -> partial slot
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
-    const int C = a.C, Cq = a.Cq, NT = CM * (CM + 1) / 2, NB = NT + CM;
+    const int C = a.C, NT = CM * (CM + 1) / 2, NB = NT + CM;
     float *buf = reinterpret_cast<float *>(smem_raw + NV * 32 * sizeof(uint16_t)) +
                  warp * ((NB + 4) / 4 * 4);
     // Tile (m, n) holds the products of feature rows 2 m (values 0, 1) and 2 m + 1 (2, 3) with
@@ -126,12 +158,12 @@ __global__ void __launch_bounds__(mma_warps(CH) * kWarp, 1)
     for (int q = lane; q < NB; q += 32) buf[q] = 0.f;  // rows and columns from C on stay zero
     __syncthreads();
 
-    bool in[CH], inq[CH];
+    bool in[CH], inq[CH];  // the lane's columns of a chunk exist in this / the previous subset
     unsigned is_res = 0u;  // bit j: the lane's feature j is column C of H' (r_hat)
 #pragma unroll
     for (int q = 0; q < CH; ++q) {
         in[q] = 32 * q + 4 * g < CM;
-        inq[q] = 32 * q + 4 * g < Cq;
+        inq[q] = 32 * q + 4 * g < a.Cq;
 #pragma unroll
         for (int u = 0; u < 4; ++u)
             if (32 * q + 4 * g + u == C) is_res |= 1u << (4 * q + u);
@@ -141,9 +173,9 @@ __global__ void __launch_bounds__(mma_warps(CH) * kWarp, 1)
     u64 acc[TILES][2];
 #pragma unroll
     for (int k = 0; k < TILES; ++k) acc[k][0] = acc[k][1] = 0ull;
-    float own_old[J], own_prev[J];
+    u64 own_old[J / 2], own_prev[J / 2];  // own row: old columns, and prev ones negated
 #pragma unroll
-    for (int j = 0; j < J; ++j) own_old[j] = own_prev[j] = 0.f;
+    for (int j = 0; j < J / 2; ++j) own_old[j] = own_prev[j] = 0ull;
 
     for (;;) {
         unsigned long long tk = 0;
@@ -176,15 +208,17 @@ __global__ void __launch_bounds__(mma_warps(CH) * kWarp, 1)
         for (;;) {
             if (FIRST && fresh) {
                 const float *z = a.Zn + (int64_t)a.rank_n[item.row] * W + 4 * g;
+                const u64 sign = 0x8000000080000000ull;
 #pragma unroll
                 for (int q = 0; q < CH; ++q) {
-                    float x[4];
-                    unpack4(ld4(z + CM + 32 * q, in[q]), x);
+                    u64 o[2], p[2];
+                    ld4(z + CM + 32 * q, in[q], p);
+                    ld4(z + 2 * CM + 32 * q, in[q], o);
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) own_prev[4 * q + u] = x[u];
-                    unpack4(ld4(z + 2 * CM + 32 * q, in[q]), x);
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) own_old[4 * q + u] = x[u];
+                    for (int u = 0; u < 2; ++u) {
+                        own_prev[2 * q + u] = p[u] ^ sign;
+                        own_old[2 * q + u] = o[u];
+                    }
                 }
             }
             // the next step's entries
@@ -205,32 +239,38 @@ __global__ void __launch_bounds__(mma_warps(CH) * kWarp, 1)
             float h[E][J], d[E];
 #pragma unroll
             for (int e = 0; e < E; ++e) {
-                d[e] = 0.f;
                 const bool valid = i0[e] >= 0;
                 const float *z0 = Z0 + (int64_t)(valid ? i0[e] : 0) * W;
                 const float *z1 = Z1 + (int64_t)(valid ? i1[e] : 0) * W;
+                u64 da = 0ull, db = 0ull;
 #pragma unroll
                 for (int q = 0; q < CH; ++q) {
-                    const bool ok = valid && in[q];
-                    float x0[4], x1[4];
-                    unpack4(ld4(z0 + 32 * q, ok), x0);
-                    unpack4(ld4(z1 + 32 * q, ok), x1);
+                    u64 x0[2], x1[2];
+                    const bool ok = valid && in[q], okq = valid && inq[q];
+                    ld4(z0 + 32 * q, ok, x0);
+                    ld4(z1 + 32 * q, ok, x1);
                     if (FIRST) {
-                        float o0[4], o1[4], p0[4], p1[4];
-                        if (NLO > 0) unpack4(ld4(z0 + 2 * CM + 32 * q, ok), o0);
-                        if (NLO > 1) unpack4(ld4(z1 + 2 * CM + 32 * q, ok), o1);
-                        unpack4(ld4(z0 + CM + 32 * q, valid && inq[q]), p0);
-                        unpack4(ld4(z1 + CM + 32 * q, valid && inq[q]), p1);
+                        u64 o0[2], o1[2], p0[2], p1[2];
+                        if (NLO > 0) ld4(z0 + 2 * CM + 32 * q, ok, o0);
+                        if (NLO > 1) ld4(z1 + 2 * CM + 32 * q, ok, o1);
+                        ld4(z0 + CM + 32 * q, okq, p0);  // zero from Cq on
+                        ld4(z1 + CM + 32 * q, okq, p1);
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const float b0 = NLO > 0 ? o0[u] : x0[u], b1 = NLO > 1 ? o1[u] : x1[u];
-                            d[e] += own_old[4 * q + u] * (b0 * b1);
-                            d[e] -= own_prev[4 * q + u] * (p0[u] * p1[u]);
+                        for (int u = 0; u < 2; ++u) {
+                            da = fma2(own_old[2 * q + u],
+                                      mul2(NLO > 0 ? o0[u] : x0[u], NLO > 1 ? o1[u] : x1[u]), da);
+                            db = fma2(own_prev[2 * q + u], mul2(p0[u], p1[u]), db);
                         }
                     }
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) h[e][4 * q + u] = x0[u] * x1[u];
+                    for (int u = 0; u < 2; ++u) {
+                        halves(mul2(x0[u], x1[u]), h[e][4 * q + 2 * u], h[e][4 * q + 2 * u + 1]);
+                    }
                 }
+                float s0, s1, r0, r1;
+                halves(da, s0, s1);
+                halves(db, r0, r1);
+                d[e] = (s0 + s1) + (r0 + r1);
             }
             if (FIRST) {
 #pragma unroll
@@ -260,13 +300,13 @@ __global__ void __launch_bounds__(mma_warps(CH) * kWarp, 1)
                 for (int m = 0; m < J / 2; ++m)
 #pragma unroll
                     for (int n = 0; n < 2 * m + 2; ++n) {
-                        float s[4] = {0.f, 0.f, 0.f, 0.f}, r[4] = {0.f, 0.f, 0.f, 0.f};
+                        float s[4], r[4];
                         const int j = 2 * m, k = m * (m + 1) + n;
                         auto mul = [&](float (&d)[4], uint32_t (&x)[J][2], uint32_t (&y)[J][2]) {
                             mma16(d, x[j][0], x[j + 1][0], x[j][1], x[j + 1][1], y[n][0], y[n][1]);
                         };
-                        mul(s, b1, b1);
-                        mul(r, b3, b1);
+                        mma16z(s, b1[j][0], b1[j + 1][0], b1[j][1], b1[j + 1][1], b1[n][0], b1[n][1]);
+                        mma16z(r, b3[j][0], b3[j + 1][0], b3[j][1], b3[j + 1][1], b1[n][0], b1[n][1]);
                         mul(r, b1, b3);
                         mul(r, b2, b2);
                         mul(r, b2, b1);
@@ -288,9 +328,9 @@ __global__ void __launch_bounds__(mma_warps(CH) * kWarp, 1)
                 for (int m = 0; m < J / 2; ++m)
 #pragma unroll
                     for (int n = 0; n < 2 * m + 2; ++n) {
-                        float s[4] = {0.f, 0.f, 0.f, 0.f};
+                        float s[4];
                         const int j = 2 * m, k = m * (m + 1) + n;
-                        mma8(s, lo[0][j], lo[0][j + 1], lo[1][j], lo[1][j + 1], h[0][n], h[1][n]);
+                        mma8z(s, lo[0][j], lo[0][j + 1], lo[1][j], lo[1][j + 1], h[0][n], h[1][n]);
                         mma8(s, h[0][j], h[0][j + 1], h[1][j], h[1][j + 1], lo[0][n], lo[1][n]);
                         mma8(s, h[0][j], h[0][j + 1], h[1][j], h[1][j + 1], h[0][n], h[1][n]);
                         acc[k][0] = add2(acc[k][0], s[0], s[1]);
