@@ -19,6 +19,7 @@
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 
 #include "sweep.cuh"
 
@@ -264,6 +265,9 @@ __device__ __forceinline__ void write_row(const PassArgs<T> &a, int row, const T
 // SM's L1, which serves the gathers of the hot (high-degree) slice rows; deeper rings
 // and explicit row caches measured slower on Zipf-skewed tensors.
 
+// SLOTS (row slots per warp): kRowSlots, or 1 where rings of four staged modes would leave few
+// warps on an SM; a step's rows are then gathered when it comes up and the other warps hide
+// the wait (mode_pass_plan_cm).
 constexpr int kLeadRows = 1;
 constexpr int kLeadIdx = 2;
 constexpr int kRowSlots = kLeadRows + 1;
@@ -353,14 +357,14 @@ struct PipeGeo {
     static __host__ __device__ size_t heads_bytes(int no) {
         return align16((size_t)(no > 0 ? no : 1) * 4);
     }
-    static __host__ __device__ size_t warp_bytes(int no, int n_lo) {
-        return kRowSlots * (rows_bytes(no, n_lo) + heads_bytes(no)) +
+    static __host__ __device__ size_t warp_bytes(int no, int n_lo, int slots = kRowSlots) {
+        return slots * (rows_bytes(no, n_lo) + heads_bytes(no)) +
                kIdxSlots * (ridx_bytes(no) + RV_BYTES + OWN_BYTES + sizeof(Step)) + OWN_BYTES;
     }
 };
 
 // Warp-private views of the ring (slot pointers are computed, not stored in arrays).
-template <class T, int CM, int NV_LO, int NV_HI>
+template <class T, int CM, int NV_LO, int NV_HI, int SLOTS = kRowSlots>
 struct PipeSmem {
     using PG = PipeGeo<T, CM, NV_LO, NV_HI>;
     unsigned char *rows0, *heads0, *ridx0, *rv0, *ownr0, *steps0;
@@ -371,8 +375,8 @@ struct PipeSmem {
         heads_b = (unsigned)PG::heads_bytes(no);
         ridx_b = (unsigned)PG::ridx_bytes(no);
         rows0 = base;
-        heads0 = rows0 + kRowSlots * rows_b;
-        ridx0 = heads0 + kRowSlots * heads_b;
+        heads0 = rows0 + SLOTS * rows_b;
+        ridx0 = heads0 + SLOTS * heads_b;
         rv0 = ridx0 + kIdxSlots * ridx_b;
         ownr0 = rv0 + kIdxSlots * PG::RV_BYTES;
         own = reinterpret_cast<T *>(ownr0 + kIdxSlots * PG::OWN_BYTES);
@@ -471,26 +475,52 @@ __device__ __forceinline__ int run_head(uint32_t heads, int lane) {
     return 31 - __clz(upto);
 }
 
-// End of an item: warp-sum (B, c) with butterflies and store them in the item's
-// partial slot (the solves run afterwards, all rows in parallel: k_solve_rows).  Lane k stores values k, k + 32, ...; the summation order is fixed.
+// End of an item: the warp's sums of (B, c) to the item's partial slot (the solves run
+// afterwards, all rows in parallel: k_solve_rows).  A reduce-scatter by halving exchanges
+// (lane distances 16 .. 1): 67 shuffles for C = 10 where a butterfly per value took 325, with
+// the same additions in the same order; lane segments of the packed values are written.  Rows
+// of few entries spend much of their step here (five-way, five entries a row: 1,900 warp
+// instructions per item before).
 template <class T, int CM>
 __device__ __forceinline__ void finish_item(const PassArgs<T> &a, const Step &s,
                                             T (&Bacc)[CM * (CM + 1) / 2], T (&cacc)[CM],
                                             int lane) {
     constexpr int NT = CM * (CM + 1) / 2, NB = NT + CM;
+    constexpr int L1 = (NB + 1) / 2, L2 = (L1 + 1) / 2, L3 = (L2 + 1) / 2, L4 = (L3 + 1) / 2,
+                  L5 = (L4 + 1) / 2;
     T *p = a.partials + (int64_t)a.items[s.it].slot * NB;
+    T f[NB];
 #pragma unroll
-    for (int v = 0; v < NT; ++v) {
-        const T tot = warp_sum(Bacc[v]);
-        if ((v & 31) == lane) p[v] = tot;
-        Bacc[v] = T(0);
-    }
+    for (int v = 0; v < NB; ++v) f[v] = v < NT ? Bacc[v < NT ? v : 0] : cacc[v < NT ? 0 : v - NT];
+    int base = 0, cnt = NB;  // the lane's segment of the sums, in f[0 .. cnt)
+    auto level = [&](auto nconst, auto hconst, int o) {
+        constexpr int n = decltype(nconst)::value, hh = decltype(hconst)::value;
+        const bool up = (lane & o) != 0;
 #pragma unroll
-    for (int c = 0; c < CM; ++c) {
-        const T tot = warp_sum(cacc[c]);
-        if (((NT + c) & 31) == lane) p[NT + c] = tot;
-        cacc[c] = T(0);
-    }
+        for (int k = 0; k < hh; ++k) {
+            const T lo = f[k], hi = k + hh < n ? f[k + hh < n ? k + hh : 0] : T(0);
+            const T send = up ? lo : hi, keep = up ? hi : lo;
+            f[k] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, o);
+        }
+        if (up) {
+            base += hh;
+            cnt = cnt > hh ? cnt - hh : 0;
+        } else {
+            cnt = cnt < hh ? cnt : hh;
+        }
+    };
+    level(std::integral_constant<int, NB>{}, std::integral_constant<int, L1>{}, 16);
+    level(std::integral_constant<int, L1>{}, std::integral_constant<int, L2>{}, 8);
+    level(std::integral_constant<int, L2>{}, std::integral_constant<int, L3>{}, 4);
+    level(std::integral_constant<int, L3>{}, std::integral_constant<int, L4>{}, 2);
+    level(std::integral_constant<int, L4>{}, std::integral_constant<int, L5>{}, 1);
+#pragma unroll
+    for (int k = 0; k < L5; ++k)
+        if (k < cnt) p[base + k] = f[k];
+#pragma unroll
+    for (int v = 0; v < NT; ++v) Bacc[v] = T(0);
+#pragma unroll
+    for (int c = 0; c < CM; ++c) cacc[c] = T(0);
 }
 
 // Per-entry arithmetic of the mode pass on staged rows.  rowp[t] points at the staged
@@ -593,12 +623,13 @@ __device__ __forceinline__ void entry_products(const T *const (&rowp)[(NO > 0 ? 
 //   c.item_begin(sm, step, idx_slot)   first step of an item (own row is in the ring)
 //   c.entry(sm, step, row_slot, idx_slot, lane)
 //   c.item_end(step)                   last step of an item
-template <class T, int CM, int NV_LO, int NV_HI, int NO, class Consumer>
+template <class T, int CM, int NV_LO, int NV_HI, int NO, int SLOTS, class Consumer>
 __device__ __forceinline__ void run_bin(const tf_item *items, int64_t it0, int64_t it1,
                                         const OtherModes<T, NO> &om, const T *res, const T *Zn,
                                         const int32_t *rank_n, int n_lo, int own_off, int own_len,
                                         bool fetch_rows,
-                                        PipeSmem<T, CM, NV_LO, NV_HI> &sm, Consumer &cons,
+                                        PipeSmem<T, CM, NV_LO, NV_HI, SLOTS> &sm,
+                                        Consumer &cons,
                                         int lane) {
     // prologue: steps 0 .. kLeadIdx-1 (indices), then rows of steps 0 .. kLeadRows-1
     Step gen = step_at_item(items, it0, it1);
@@ -612,6 +643,31 @@ __device__ __forceinline__ void run_bin(const tf_item *items, int64_t it0, int64
     cp_async_commit();
     cp_async_wait<0>();
     __syncwarp();
+    if constexpr (SLOTS == 1) {
+        for (int is = 0;; is = (is + 1) % kIdxSlots) {
+            const Step cur = *sm.step(is);
+            if (!(cur.flags & 1)) break;
+            if (fetch_rows)
+                issue_rows<T, CM, NV_LO, NV_HI, NO>(cur, sm.rows(0), sm.heads(0), sm.ridx(is), om,
+                                                    n_lo, lane);
+            cp_async_commit();
+            const int ia = (is + kLeadIdx) % kIdxSlots;
+            if (lane == 0) *sm.step(ia) = gen;
+            issue_idx<T, CM, NO>(gen, sm.ridx(ia), sm.rv(ia), sm.ownring(ia), om, res, items, Zn,
+                                 rank_n, own_off, own_len, lane);
+            gen = step_next(gen, items, it1);
+            cp_async_commit();
+            cp_async_wait<1>();  // this step's rows, and the next one's indices
+            __syncwarp();
+            if (cur.flags & 2) cons.item_begin(sm, cur, is, lane);
+            cons.entry(sm, cur, 0, is, lane);
+            if (cur.flags & 4) cons.item_end(cur, lane);
+            __syncwarp();
+        }
+        cp_async_wait<0>();
+        __syncwarp();
+        return;
+    }
 #pragma unroll
     for (int k = 0; k < kLeadRows; ++k) {
         if (fetch_rows) {
@@ -654,13 +710,13 @@ __device__ __forceinline__ void run_bin(const tf_item *items, int64_t it0, int64
     __syncwarp();
 }
 
-template <class T, int CM, int NO, bool FIRST>
+template <class T, int CM, int NO, bool FIRST, int SLOTS>
 struct PassConsumer {
     using G = Geo<T, CM>;
     static constexpr int NV_LO = FIRST ? G::NV_ALL : G::NV_CUR;  // cur|prev|old
     static constexpr int NV_HI = FIRST ? G::NV_CP : G::NV_CUR;   // cur|prev
     using PG = PipeGeo<T, CM, NV_LO, NV_HI>;
-    using SM = PipeSmem<T, CM, NV_LO, NV_HI>;
+    using SM = PipeSmem<T, CM, NV_LO, NV_HI, SLOTS>;
     const PassArgs<T> &a;
     int no, n_lo;
     T Bacc[G::NT], cacc[CM];
@@ -735,10 +791,10 @@ __device__ __forceinline__ OtherModes<T, NO> other_modes(const int32_t *const *p
 
 // Bytes of one warp's ring for a mode pass of mode n (n_lo = n other modes before it).
 template <class T, int CM, bool FIRST>
-__host__ __device__ size_t pass_warp_bytes(int N, int n) {
+__host__ __device__ size_t pass_warp_bytes(int N, int n, int slots) {
     using G = Geo<T, CM>;
     using PG = PipeGeo<T, CM, FIRST ? G::NV_ALL : G::NV_CUR, FIRST ? G::NV_CP : G::NV_CUR>;
-    return PG::warp_bytes(N - 1, n);
+    return PG::warp_bytes(N - 1, n, slots);
 }
 
 // Warps per block of the mode pass (one block per SM): as many as the registers of the
@@ -752,17 +808,17 @@ constexpr int pass_max_warps() {
 // FIRST: the split's first inner iteration (R-hat refresh) or a later one.
 // One block per SM (the staging rings are small, so most of the SM's shared memory
 // stays L1 cache: the hottest slice rows are served from there).
-template <class T, int CM, int NO, bool FIRST>
+template <class T, int CM, int NO, bool FIRST, int SLOTS>
 __global__ void __launch_bounds__(pass_max_warps<T, CM>() * kWarp, 1)
     k_mode_pass(const PassArgs<T> a) {
-    using Cons = PassConsumer<T, CM, NO, FIRST>;
+    using Cons = PassConsumer<T, CM, NO, FIRST, SLOTS>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ const int32_t *s_oidx[kMaxModes - 1];
     __shared__ const T *s_Zo[kMaxModes - 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const OtherModes<T, NO> om = other_modes<T, NO>(a.oidx, a.Zo, a.N, s_oidx, s_Zo);
     const int no = a.N - 1, n_lo = a.n;
-    typename Cons::SM sm(smem_raw + warp * pass_warp_bytes<T, CM, FIRST>(a.N, a.n), no, n_lo);
+    typename Cons::SM sm(smem_raw + warp * pass_warp_bytes<T, CM, FIRST>(a.N, a.n, SLOTS), no, n_lo);
     Cons cons(a, no, n_lo);
     // own row: prev|old regions, [CM, 3 CM) of the own slice row (first iteration only)
     const int own_len = FIRST ? 2 * CM : 0;
@@ -774,7 +830,7 @@ __global__ void __launch_bounds__(pass_max_warps<T, CM>() * kWarp, 1)
         tk = __shfl_sync(0xFFFFFFFFu, tk, 0);
         if (tk >= (unsigned long long)a.P) break;
         const int bin = (int)tk;
-        run_bin<T, CM, Cons::NV_LO, Cons::NV_HI, NO>(a.items, a.bin_ptr[bin], a.bin_ptr[bin + 1],
+        run_bin<T, CM, Cons::NV_LO, Cons::NV_HI, NO, SLOTS>(a.items, a.bin_ptr[bin], a.bin_ptr[bin + 1],
                                                      om, a.res, a.Zn, a.rank_n, n_lo, CM, own_len,
                                                      true, sm, cons, lane);
     }
@@ -1053,7 +1109,7 @@ __global__ void __launch_bounds__(kPassThreads) k_res(const ResArgs<T> a) {
     Cons cons(a, no);
     const int bin = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (bin < a.P)
-        run_bin<T, CM, Cons::NV_LO, Cons::NV_HI, 0>(a.items, a.bin_ptr[bin], a.bin_ptr[bin + 1], om,
+        run_bin<T, CM, Cons::NV_LO, Cons::NV_HI, 0, kRowSlots>(a.items, a.bin_ptr[bin], a.bin_ptr[bin + 1], om,
                                                     a.res, a.Zn, a.rank_n, no, 0, a.Cq > 0 ? CM : 0,
                                                     a.Cq > 0, sm, cons, lane);
     if (a.what != 0) return;
@@ -1090,33 +1146,49 @@ inline int best_warps_per_block(size_t warp_bytes) {
 // Three- and five-way tensors get the number of other modes as a compile-time constant
 // (fully unrolled mode loops); other orders run the generic kernel.
 template <class T, int CM>
-auto mode_pass_kernel(int N, bool first) {
-    if (N == 3) return first ? k_mode_pass<T, CM, 2, true> : k_mode_pass<T, CM, 2, false>;
+auto mode_pass_kernel(int N, bool first, int slots) {
+    constexpr int S = kRowSlots;
+    if (N == 3) return first ? k_mode_pass<T, CM, 2, true, S> : k_mode_pass<T, CM, 2, false, S>;
     if constexpr (sizeof(T) == 4)
-        if (N == 5) return first ? k_mode_pass<T, CM, 4, true> : k_mode_pass<T, CM, 4, false>;
-    return first ? k_mode_pass<T, CM, 0, true> : k_mode_pass<T, CM, 0, false>;
+        if (N == 5) {
+            if (slots == 1)
+                return first ? k_mode_pass<T, CM, 4, true, 1> : k_mode_pass<T, CM, 4, false, 1>;
+            return first ? k_mode_pass<T, CM, 4, true, S> : k_mode_pass<T, CM, 4, false, S>;
+        }
+    return first ? k_mode_pass<T, CM, 0, true, S> : k_mode_pass<T, CM, 0, false, S>;
 }
 
 // Plan of a mode-n pass: one block per SM with as many warps as fit (up to
-// pass_max_warps); the shared memory the rings leave is L1 cache.
+// pass_max_warps); the shared memory the rings leave is L1 cache.  Float five-way tensors
+// take one row slot per warp where two would leave fewer than pass_max_warps: C = 10, modes
+// of 1e6 rows, 2e7 entries, passes with 9 to 5 warps of two slots 3.5 to 5.1 ms, 2.35 to 2.8
+// ms with 12 to 10 warps of one (and the cheaper ends of items, finish_item).
 template <class T, int CM, bool FIRST>
 PassPlan mode_pass_plan_cm(int N, int n, int num_sms, int P) {
     constexpr size_t kReserve = 1024;  // static shared memory of the kernel
     int dev = 0, smem_blk = 0;
     TFS_CUDA(cudaGetDevice(&dev));
     TFS_CUDA(cudaDeviceGetAttribute(&smem_blk, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    const size_t ring = pass_warp_bytes<T, CM, FIRST>(N, n);
     PassPlan plan;
-    plan.warps = (int)std::min<size_t>(pass_max_warps<T, CM>(), ((size_t)smem_blk - kReserve) / ring);
+    const size_t room = (size_t)smem_blk - kReserve;
+    auto fit = [&](int slots) {
+        return (int)std::min<size_t>(pass_max_warps<T, CM>(),
+                                     room / pass_warp_bytes<T, CM, FIRST>(N, n, slots));
+    };
+    plan.warps = fit(kRowSlots);
+    if (sizeof(T) == 4 && N == 5 && fit(1) > plan.warps) {
+        plan.slots = 1;
+        plan.warps = fit(1);
+    }
     if (plan.warps < 1) throw ApiError{TF_EINVAL, "mode pass does not fit in shared memory"};
-    plan.smem = (size_t)plan.warps * ring;
+    plan.smem = (size_t)plan.warps * pass_warp_bytes<T, CM, FIRST>(N, n, plan.slots);
     plan.grid = std::max(1, std::min(num_sms, (P + plan.warps - 1) / plan.warps));
     return plan;
 }
 
 template <class T, int CM>
 void launch_mode_pass_cm(const PassArgs<T> &a, const PassPlan &plan, cudaStream_t st) {
-    auto kern = mode_pass_kernel<T, CM>(a.N, a.first != 0);
+    auto kern = mode_pass_kernel<T, CM>(a.N, a.first != 0, plan.slots);
     TFS_CUDA(raise_smem_limit((const void *)kern, (int)plan.smem));
     kern<<<plan.grid, plan.warps * kWarp, plan.smem, st>>>(a);
     TFS_CUDA(cudaGetLastError());

@@ -237,6 +237,7 @@ struct SolveRows {
 // Launch plan of one cp.async mode pass: one block per SM, warps per block.
 struct PassPlan {
     int warps = 0, grid = 0;
+    int slots = 2;  // row slots per warp (mode_pass.cuh)
     size_t smem = 0;
 };
 // Wide pass of float three-way tensors for C <= 63 (mma_pass.cu); the plan has no dynamic
