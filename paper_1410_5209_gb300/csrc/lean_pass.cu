@@ -661,7 +661,12 @@ LeanPlan lean_pass_plan(int CM, bool first, int n, const int64_t *dims_o,
     const int fit = (int)std::min<size_t>(max_warps, ((size_t)smem_blk - kStatic) / warp_bytes);
     if (fit < 1) throw ApiError{TF_EINVAL, "lean mode pass: staging pool does not fit"};
     pl.warps = std::max(1, std::min(warps > 0 ? warps : max_warps, fit));
-    const size_t ring_bytes = (size_t)pl.warps * warp_bytes;
+    const int full_warps = pl.warps;
+    // fewer bins than warps: spread them over the SMs (60,000 entries, 937 bins, C = 4: 47
+    // blocks of 20 warps before; with the next rule the three passes 12.6 / 9.5 / 13.4 us
+    // before, 9.1 / 8.9 / 10.6 now)
+    if (warps <= 0) pl.warps = std::min(pl.warps, std::max(1, (P + num_sms - 1) / num_sms));
+    const size_t ring_bytes = (size_t)full_warps * warp_bytes;
     const size_t avail =
         (size_t)smem_blk > ring_bytes + kStatic ? smem_blk - ring_bytes - kStatic : 0;
     // cache rows: greedy in chunks of 32 rows by entries covered per byte, the run mode's
@@ -699,13 +704,32 @@ LeanPlan lean_pass_plan(int CM, bool first, int n, const int64_t *dims_o,
         const std::vector<int64_t> &dc = *deg_cum[var];
         pl.coverage = nnz > 0 ? (double)dc[R[var]] / (double)nnz : 1.0;
     }
+    pl.grid = std::max(1, std::min(num_sms, (P + pl.warps - 1) / pl.warps));
+    // every block copies the cached rows: a row with fewer entries than there are blocks is
+    // gathered less often than it would be copied (rows are in decreasing order of entries;
+    // the device's SM count, so that an SM limit does not change the gather plan)
+    int dev_sms = 0;
+    TFS_CUDA(cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, dev));
+    const int blocks = std::min(dev_sms, P);
+    if (max_cache_rows < 0)
+        for (int t = 0; t < 2; ++t) {
+            const std::vector<int64_t> &dc = *deg_cum[t];
+            int lo = 0, hi = R[t];
+            while (lo < hi) {
+                const int mid = (lo + hi) / 2;
+                if (dc[mid + 1] - dc[mid] >= blocks)
+                    lo = mid + 1;
+                else
+                    hi = mid;
+            }
+            R[t] = lo;
+        }
     lp.R[0] = R[0];
     lp.R[1] = R[1];
     lp.cache_off[0] = 0;
     lp.cache_off[1] = R[0] * cs[0];
     lp.ring_off = (lp.cache_off[1] + R[1] * cs[1] + 3) / 4 * 4;
     pl.smem = (size_t)(lp.ring_off + pl.warps * lp.ring_floats) * 4;
-    pl.grid = std::max(1, std::min(num_sms, (P + pl.warps - 1) / pl.warps));
     return pl;
 }
 

@@ -836,6 +836,91 @@ __global__ void __launch_bounds__(pass_max_warps<T, CM>() * kWarp, 1)
     }
 }
 
+// Mode pass of three-way tensors for C = 1 (CDTF): a slice row is one 16-byte vector (32 bytes
+// for doubles) of cur, prev and old, so each lane reads its entries' rows directly, four
+// entries in flight, instead of staging them for the warp; lane and entry pairing and every
+// sum are those of the staged pass.  Bound: the row gathers (L1 lookups, one line per lane).
+// 1e7 entries, modes of 30,011 / 20,021 / 503 rows: 0.112 ms a pass staged, 0.060 now.
+template <class T>
+struct RowOne {
+    T cur, prev, old;
+};
+template <class T, bool ALL>
+__device__ __forceinline__ RowOne<T> load_row_one(const T *z) {
+    RowOne<T> r{};
+    if constexpr (!ALL) {
+        r.cur = z[0];
+    } else if constexpr (sizeof(T) == 4) {
+        const float4 v = *reinterpret_cast<const float4 *>(z);
+        r.cur = v.x, r.prev = v.y, r.old = v.z;
+    } else {
+        const double2 v = *reinterpret_cast<const double2 *>(z);
+        r.cur = v.x, r.prev = v.y, r.old = z[2];
+    }
+    return r;
+}
+
+constexpr int kOneWarps = 32;
+
+template <class T, bool FIRST>
+__global__ void __launch_bounds__(kOneWarps * kWarp, 1) k_pass_one(const PassArgs<T> a) {
+    constexpr int W = Geo<T, 1>::W, U = 4;
+    const int lane = threadIdx.x & 31, n_lo = a.n, Cq = a.Cq;
+    const T *Z0 = a.Zo[0], *Z1 = a.Zo[1];
+    const int32_t *ix0 = a.oidx[0], *ix1 = a.oidx[1];
+    for (;;) {
+        unsigned long long tk = 0;
+        if (lane == 0) tk = atomicAdd(a.ticket, 1ull) - a.ticket_base;
+        tk = __shfl_sync(0xFFFFFFFFu, tk, 0);
+        if (tk >= (unsigned long long)a.P) break;
+        for (int64_t it = a.bin_ptr[tk]; it < a.bin_ptr[tk + 1]; ++it) {
+            const tf_item item = a.items[it];
+            RowOne<T> own{};
+            if (FIRST) own = load_row_one<T, true>(a.Zn + (int64_t)a.rank_n[item.row] * W);
+            T B[1] = {T(0)}, c[1] = {T(0)};
+            const int end = (int)(item.begin + item.len);  // nnz < 2^31
+            for (int j = (int)item.begin + lane; j - lane < end; j += U * kWarp) {
+                int32_t i0[U], i1[U];
+                T rv[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const bool in = j + u * kWarp < end;
+                    i0[u] = in ? ix0[j + u * kWarp] : -1;
+                    i1[u] = in ? ix1[j + u * kWarp] : 0;
+                    rv[u] = in ? a.res[j + u * kWarp] : T(0);
+                }
+                RowOne<T> r0[U], r1[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    r0[u] = load_row_one<T, FIRST>(Z0 + (int64_t)(i0[u] < 0 ? 0 : i0[u]) * W);
+                    r1[u] = load_row_one<T, FIRST>(Z1 + (int64_t)i1[u] * W);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (i0[u] < 0) continue;
+                    const T h = r0[u].cur * r1[u].cur;
+                    T v = rv[u];
+                    if (FIRST) {
+                        T pp = T(0), po = T(0);
+                        if (Cq > 0) pp += own.prev * (r0[u].prev * r1[u].prev);
+                        if (n_lo == 0)
+                            po += own.old * h;
+                        else
+                            po += own.old * (r0[u].old * (n_lo > 1 ? r1[u].old : r1[u].cur));
+                        v = v - pp + po;
+                        a.res[j + u * kWarp] = v;
+                    }
+                    c[0] += v * h;
+                    B[0] += h * h;
+                }
+            }
+            Step st{};
+            st.it = (int32_t)it;
+            finish_item<T, 1>(a, st, B, c, lane);
+        }
+    }
+}
+
 // Row solves of a mode: (B + lambda I) a = c (Eq. 4) for every row, by the register Cholesky
 // of Section 3.1 with one lane per row, in one launch.  A row with several slots is summed as
 // G = kSlotSums / NB sums of every G-th slot, added in order (plain order up to G slots).
@@ -1044,12 +1129,13 @@ __global__ void __launch_bounds__(kSolveThreads) k_solve_rows(const PassArgs<T> 
 // split's final values): r = res - sum_{c < Cq} prod_l Z_l[i_l, c].  One warp per bin,
 // every bin launched (the per-block double sums are then in a fixed order); the same
 // warp pipeline as the mode pass feeds it.
-template <class T, int CM>
+template <class T, int CM, int NO>
 struct ResConsumer {
     using G = Geo<T, CM>;
     static constexpr int NV_LO = G::NV_CUR, NV_HI = G::NV_CUR;
+    static constexpr int SLOTS = NO > 2 ? 1 : kRowSlots;  // as the passes of four other modes
     using PG = PipeGeo<T, CM, NV_LO, NV_HI>;
-    using SM = PipeSmem<T, CM, NV_LO, NV_HI>;
+    using SM = PipeSmem<T, CM, NV_LO, NV_HI, SLOTS>;
     const ResArgs<T> &a;
     int no;
     double acc = 0.0;
@@ -1069,7 +1155,8 @@ struct ResConsumer {
             const uint32_t *hd = sm.heads(rs);
             T q[CM], x[CM];
             lds_range<T, 0, CM>(q, sm.own);
-            for (int t = 0; t < no; ++t) {
+#pragma unroll(NO > 0 ? NO : 1)
+            for (int t = 0; t < (NO > 0 ? NO : no); ++t) {
                 lds_range<T, 0, CM>(x, slot + PG::mode_off(t, no) + run_head(hd[t], lane) * PG::RS_LO);
 #pragma unroll
                 for (int c = 0; c < CM; ++c) q[c] *= x[c];
@@ -1089,29 +1176,35 @@ struct ResConsumer {
     __device__ __forceinline__ void item_end(const Step &, int) {}
 };
 
+// Number of other modes as a compile-time constant: five-way float tensors, any (0).
+template <class T>
+__host__ __device__ constexpr int res_no(int N) {
+    return sizeof(T) == 4 && N == 5 ? 4 : 0;
+}
 template <class T, int CM>
 __host__ __device__ size_t res_warp_bytes(int N) {
     using G = Geo<T, CM>;
-    return PipeGeo<T, CM, G::NV_CUR, G::NV_CUR>::warp_bytes(N - 1, N - 1);
+    return PipeGeo<T, CM, G::NV_CUR, G::NV_CUR>::warp_bytes(N - 1, N - 1,
+                                                            res_no<T>(N) > 2 ? 1 : kRowSlots);
 }
 
-template <class T, int CM>
+template <class T, int CM, int NO>
 __global__ void __launch_bounds__(kPassThreads) k_res(const ResArgs<T> a) {
-    using Cons = ResConsumer<T, CM>;
+    using Cons = ResConsumer<T, CM, NO>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double wsum[kPassThreads / kWarp];
     __shared__ const int32_t *s_oidx[kMaxModes - 1];
     __shared__ const T *s_Zo[kMaxModes - 1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int no = a.N - 1;
-    const OtherModes<T, 0> om = other_modes<T, 0>(a.oidx, a.Zo, a.N, s_oidx, s_Zo);
+    const OtherModes<T, NO> om = other_modes<T, NO>(a.oidx, a.Zo, a.N, s_oidx, s_Zo);
     typename Cons::SM sm(smem_raw + warp * res_warp_bytes<T, CM>(a.N), no, no);
     Cons cons(a, no);
     const int bin = (int)(((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     if (bin < a.P)
-        run_bin<T, CM, Cons::NV_LO, Cons::NV_HI, 0, kRowSlots>(a.items, a.bin_ptr[bin], a.bin_ptr[bin + 1], om,
-                                                    a.res, a.Zn, a.rank_n, no, 0, a.Cq > 0 ? CM : 0,
-                                                    a.Cq > 0, sm, cons, lane);
+        run_bin<T, CM, Cons::NV_LO, Cons::NV_HI, NO, Cons::SLOTS>(
+            a.items, a.bin_ptr[bin], a.bin_ptr[bin + 1], om, a.res, a.Zn, a.rank_n, no, 0,
+            a.Cq > 0 ? CM : 0, a.Cq > 0, sm, cons, lane);
     if (a.what != 0) return;
     const double acc = warp_sum_d(cons.acc);
     if (lane == 0) wsum[warp] = acc;
@@ -1148,7 +1241,8 @@ inline int best_warps_per_block(size_t warp_bytes) {
 template <class T, int CM>
 auto mode_pass_kernel(int N, bool first, int slots) {
     constexpr int S = kRowSlots;
-    if (N == 3) return first ? k_mode_pass<T, CM, 2, true, S> : k_mode_pass<T, CM, 2, false, S>;
+    if constexpr (CM > 1)  // CM = 1: k_pass_one
+        if (N == 3) return first ? k_mode_pass<T, CM, 2, true, S> : k_mode_pass<T, CM, 2, false, S>;
     if constexpr (sizeof(T) == 4)
         if (N == 5) {
             if (slots == 1)
@@ -1170,6 +1264,11 @@ PassPlan mode_pass_plan_cm(int N, int n, int num_sms, int P) {
     TFS_CUDA(cudaGetDevice(&dev));
     TFS_CUDA(cudaDeviceGetAttribute(&smem_blk, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     PassPlan plan;
+    if (CM == 1 && N == 3) {  // k_pass_one
+        plan.warps = kOneWarps;
+        plan.grid = std::max(1, std::min(num_sms, (P + kOneWarps - 1) / kOneWarps));
+        return plan;
+    }
     const size_t room = (size_t)smem_blk - kReserve;
     auto fit = [&](int slots) {
         return (int)std::min<size_t>(pass_max_warps<T, CM>(),
@@ -1188,6 +1287,16 @@ PassPlan mode_pass_plan_cm(int N, int n, int num_sms, int P) {
 
 template <class T, int CM>
 void launch_mode_pass_cm(const PassArgs<T> &a, const PassPlan &plan, cudaStream_t st) {
+    if constexpr (CM == 1) {
+        if (a.N == 3) {
+            if (a.first)
+                k_pass_one<T, true><<<plan.grid, plan.warps * kWarp, 0, st>>>(a);
+            else
+                k_pass_one<T, false><<<plan.grid, plan.warps * kWarp, 0, st>>>(a);
+            TFS_CUDA(cudaGetLastError());
+            return;
+        }
+    }
     auto kern = mode_pass_kernel<T, CM>(a.N, a.first != 0, plan.slots);
     TFS_CUDA(raise_smem_limit((const void *)kern, (int)plan.smem));
     kern<<<plan.grid, plan.warps * kWarp, plan.smem, st>>>(a);
@@ -1224,8 +1333,11 @@ template <class T, int CM>
 void launch_res_cm(const ResArgs<T> &a, cudaStream_t st) {
     const int wpb = res_warps<T, CM>(a.N);
     const size_t smem = wpb * res_warp_bytes<T, CM>(a.N);
-    TFS_CUDA(raise_smem_limit((const void *)k_res<T, CM>, (int)smem));
-    k_res<T, CM><<<res_blocks(a.P, wpb), wpb * kWarp, smem, st>>>(a);
+    auto kern = k_res<T, CM, 0>;
+    if constexpr (res_no<T>(5) == 4)
+        if (a.N == 5) kern = k_res<T, CM, 4>;
+    TFS_CUDA(raise_smem_limit((const void *)kern, (int)smem));
+    kern<<<res_blocks(a.P, wpb), wpb * kWarp, smem, st>>>(a);
     TFS_CUDA(cudaGetLastError());
 }
 

@@ -101,19 +101,44 @@ __global__ void __launch_bounds__(kResThreads) k_init_res(const InitArgs<T> a) {
     }
 }
 
+// Sum of squares of a factor matrix, each row weighted by its entries if off is given; one
+// double per block.  Float values: squares and sums as pairs of floats (float_pair.cuh; in
+// FP64 the conversions and sums bound it), with the FP64 form for a thread whose largest value
+// lies outside 2^-40 .. 2^50.  Without weights the matrix is one flat array; with them a
+// thread takes a row at a time.
+template <class T>
+__device__ __forceinline__ double sum_squares(const T *p, int64_t n, int64_t first, int64_t step) {
+    double s = 0.0;
+    if constexpr (sizeof(T) == 4) {
+        FloatPair acc = {0.f, 0.f};
+        float big = 0.f;
+        for (int64_t i = first; i < n; i += step) {
+            const float v = p[i];
+            FloatPair q;
+            q.h = two_prod(v, v, q.l);
+            pair_add(acc, q.h, q.l);
+            big = fmaxf(big, fabsf(v));
+        }
+        s = (double)acc.h + (double)acc.l;
+        if (big == 0.f || (big > 0x1p-40f && big < 0x1p50f && s == s)) return s;
+        s = 0.0;
+    }
+    for (int64_t i = first; i < n; i += step) s += (double)p[i] * (double)p[i];
+    return s;
+}
+
 template <class T>
 __global__ void __launch_bounds__(kResThreads) k_reg(const T *A, int64_t I, int K,
                                                      const int64_t *off, double *block_out) {
     __shared__ double wsum[kResThreads / kWarp];
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
+                  step = (int64_t)gridDim.x * blockDim.x;
     double acc = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < I;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int k = 0; k < K; ++k) {
-            const double v = (double)A[i * K + k];
-            s += v * v;
-        }
-        acc += off ? s * (double)(off[i + 1] - off[i]) : s;
+    if (off) {
+        for (int64_t i = first; i < I; i += step)
+            acc += sum_squares(A + i * K, K, 0, 1) * (double)(off[i + 1] - off[i]);
+    } else {
+        acc = sum_squares(A, I * K, first, step);
     }
     acc = warp_sum_d(acc);
     if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = acc;
@@ -125,10 +150,21 @@ __global__ void __launch_bounds__(kResThreads) k_reg(const T *A, int64_t I, int 
     }
 }
 
-__global__ void k_sum_blocks(const double *in, int n, double *out) {
-    __shared__ double sh[256];
+// Sum of n doubles in a fixed order, one block: 97,000 item sums took 104 us with 256 threads
+// and one load in flight each.
+constexpr int kSumThreads = 1024;
+
+__global__ void __launch_bounds__(kSumThreads) k_sum_blocks(const double *in, int n, double *out) {
+    constexpr int U = 8;
+    __shared__ double sh[kSumThreads];
     double s = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) s += in[i];
+    for (int64_t i = threadIdx.x; i < n; i += U * kSumThreads) {
+        double v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = i + u * kSumThreads < n ? in[i + u * kSumThreads] : 0.0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) s += v[u];
+    }
     sh[threadIdx.x] = s;
     __syncthreads();
     for (int w = blockDim.x / 2; w > 0; w >>= 1) {
@@ -331,7 +367,7 @@ void launch_reg(const T *A, int64_t I, int K, const int64_t *off, double *block_
 }
 
 void launch_sum_blocks(const double *in, int n, double *out, cudaStream_t st) {
-    k_sum_blocks<<<1, 256, 0, st>>>(in, n, out);
+    k_sum_blocks<<<1, kSumThreads, 0, st>>>(in, n, out);
     TFS_CUDA(cudaGetLastError());
 }
 
