@@ -738,17 +738,34 @@ struct Impl : CtxBase {
         bh.offs.assign((size_t)N, {});
         bh.ids.assign((size_t)N, {});
         bh.ranks.assign((size_t)N, {});
-        run_per_mode([&](int n) {
-            const int64_t I = dims[n];
-            const uint32_t *c = h_cnt + f.cnt_off[n];
-            std::vector<int64_t> count((size_t)I);
-            std::vector<int64_t> &off = bh.offs[n];
-            off.assign((size_t)I + 1, 0);
-            for (int64_t i = 0; i < I; ++i) {
-                count[i] = c[i];
-                off[i + 1] = off[i] + c[i];
+        // each mode on two host threads: its schedule, and its degree ranks
+        bh.plans.assign((size_t)N, {});
+        std::vector<std::exception_ptr> plan_err((size_t)N);
+        std::vector<std::thread> planners;
+        struct Joiner {
+            std::vector<std::thread> &t;
+            ~Joiner() {
+                for (auto &x : t)
+                    if (x.joinable()) x.join();
             }
-            degree_order(n, count, bh.ids[n], bh.ranks[n]);
+        } join_planners{planners};
+        for (int n = 0; n < N; ++n) {
+            const uint32_t *c = h_cnt + f.cnt_off[n];
+            std::vector<int64_t> &off = bh.offs[n];
+            off.resize((size_t)dims[n] + 1);
+            off[0] = 0;
+            for (int64_t i = 0; i < dims[n]; ++i) off[(size_t)i + 1] = off[(size_t)i] + c[i];
+            planners.emplace_back([&, n] {
+                try {
+                    bh.plans[n] = plan_host(bh.offs[n], dims[n]);
+                } catch (...) {
+                    plan_err[n] = std::current_exception();
+                }
+            });
+        }
+        run_per_mode([&](int n) {
+            const uint32_t *c = h_cnt + f.cnt_off[n];
+            degree_order(n, std::vector<int64_t>(c, c + dims[n]), bh.ids[n], bh.ranks[n]);
         });
         // page-locked staging: the copies queue behind mode 0's sort without holding the host
         for (int n = 0; n < N; ++n) {
@@ -760,26 +777,6 @@ struct Impl : CtxBase {
             bh.stage.copy(L.id_of.p, bh.ids[n].data(), L.I * sizeof(int32_t), st);
             bh.stage.copy(L.rank_of.p, bh.ranks[n].data(), L.I * sizeof(int32_t), st);
         }
-        // the schedules on host threads while the device continues
-        bh.plans.assign((size_t)N, {});
-        std::vector<std::exception_ptr> plan_err((size_t)N);
-        std::vector<std::thread> planners;
-        struct Joiner {
-            std::vector<std::thread> &t;
-            ~Joiner() {
-                for (auto &x : t)
-                    if (x.joinable()) x.join();
-            }
-        } join_planners{planners};
-        for (int n = 0; n < N; ++n)
-            planners.emplace_back([&, n] {
-                try {
-                    bh.plans[n] = plan_host(bh.offs[n], dims[n]);
-                } catch (...) {
-                    plan_err[n] = std::current_exception();
-                }
-            });
-
         for (int n = 0; n < N; ++n) {
             ModeLayout &L = mode[n];
             L.ostride = (nnz + 64 + 63) / 64 * 64;
@@ -869,18 +866,18 @@ struct Impl : CtxBase {
         PlanHost h;
         tf_status s = plan_mode(off.data(), I, P, 0, policy, seed, h.items, h.n_slots, h.bin_ptr);
         if (s != TF_OK) throw ApiError{s, "row scheduling failed"};
-        // rows and their slots (a row's slots are consecutive, in entry order):
-        std::vector<int32_t> item_of_slot((size_t)h.n_slots, -1);
-        for (size_t i = 0; i < h.items.size(); ++i) item_of_slot[(size_t)h.items[i].slot] = (int32_t)i;
-        for (int64_t q = 0; q < h.n_slots;) {
-            const tf_item &first = h.items[(size_t)item_of_slot[(size_t)q]];
-            int64_t q2 = q + 1;
-            while (q2 < h.n_slots && h.items[(size_t)item_of_slot[(size_t)q2]].row == first.row) ++q2;
-            const int64_t r = first.row;
-            const SplitRow sr{first.row, first.slot, (int32_t)(q2 - q), 0, off[r + 1] - off[r]};
-            (q2 - q > 1 ? h.split : h.single).push_back(sr);
-            q = q2;
+        // rows and their slots: consecutive, in row order (plan_mode's chunks of rows longer
+        // than its cap, one slot per row otherwise)
+        const int64_t cap = std::max<int64_t>(1, (off[I] + P - 1) / P);
+        h.single.reserve((size_t)I);
+        int32_t slot = 0;
+        for (int64_t r = 0; r < I; ++r) {
+            const int64_t len = off[r + 1] - off[r];
+            const int32_t slots = policy == TF_SCHED_LPT && len > cap ? (int32_t)((len + cap - 1) / cap) : 1;
+            (slots > 1 ? h.split : h.single).push_back({(int32_t)r, slot, slots, 0, len});
+            slot += slots;
         }
+        if (slot != h.n_slots) throw ApiError{TF_ECUDA, "row schedule and slots disagree"};
         auto upto = [&](std::vector<SplitRow>::iterator from, int slots) {
             return std::stable_partition(from, h.split.end(),
                                          [=](const SplitRow &r) { return r.n_slots <= slots; });
