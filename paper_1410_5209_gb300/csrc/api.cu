@@ -1127,8 +1127,9 @@ struct Impl : CtxBase {
         g->nsteps = std::max<int64_t>(cap_steps, 1);
         g->steps.alloc((size_t)g->nsteps * gather_plan_step_bytes(), st);
         g->step_range.alloc((size_t)2 * std::max(Pn, 1), st);
-        g->list.alloc((size_t)std::max<int64_t>(2 * nnz, 1), st);
-        g->word.alloc((size_t)std::max<int64_t>(nnz, 1), st);
+        // the pass reads whole vectors: up to 36 values from a step's aligned start
+        g->list.alloc((size_t)2 * nnz + 64, st);
+        g->word.alloc((size_t)nnz + 64, st);
         GatherPlanDev d = dev_of(*g);
         launch_gather_plan(L.items.p, L.bin_ptr.p, Pn, ixR, ixV, L.rank_of.p, RR, RV, cap, first,
                            L.plan_base.p, g->step_range.p, g->steps.p,

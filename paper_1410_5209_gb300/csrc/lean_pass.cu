@@ -147,6 +147,7 @@ struct LG {
 };
 
 constexpr int kLeanSlots = 2;        // pool slots: cold rows are staged one step ahead
+constexpr int kStream = 36;          // values of a step's stream: 32 from anywhere in a vector
 
 // ---------------------------------------------------------------------------- the pass
 // GK: how the Gram matrix and right-hand side are accumulated.  2: not at all: the loss
@@ -220,6 +221,13 @@ __global__ void __launch_bounds__(lean_max_warps(CM, GK) * kWarp, 1)
     const unsigned cacheR = saddr(sm + lp.cache_off[RUN]), cacheV = saddr(sm + lp.cache_off[VAR]);
     const unsigned ring_s = saddr(sm + lp.ring_off + warp * lp.ring_floats);
     const unsigned str_s = ring_s + 4u * (unsigned)lp.str_off;
+    // the lane's vector of a step's streams: lanes 0-8 words, 9-17 residuals, 18-26 list
+    const int str_g = lane / 9, str_q = 4 * (lane - 9 * str_g);
+    const unsigned str_dst = str_s + 4u * (unsigned)(str_g * kStream + str_q);
+    const uint32_t *str_src = (str_g == 0 ? word
+                               : str_g == 1 ? reinterpret_cast<const uint32_t *>(a.res)
+                                            : reinterpret_cast<const uint32_t *>(list)) +
+                              str_q;
 
     u64 acc[GK == 0 ? NACC : 1];
 #pragma unroll
@@ -262,6 +270,8 @@ __global__ void __launch_bounds__(lean_max_warps(CM, GK) * kWarp, 1)
             rrank = 0;
             if (base + lane < s_end) {
                 rec = steps[base + lane];
+                // where the streams' first values lie in their 16-byte vectors
+                rec.info |= ((uint32_t)rec.j0 & 3u) << 27 | (rec.list_off & 3u) << 29;
                 if (FIRST || GK == 2) rrank = srank[base + lane];
             }
         };
@@ -271,36 +281,36 @@ __global__ void __launch_bounds__(lean_max_warps(CM, GK) * kWarp, 1)
         auto info_of = [&](int s) -> uint32_t {
             return s < s_end ? __shfl_sync(0xFFFFFFFFu, rec.info, s - wb) : 0u;
         };
-        // Streams in the warp's shared-memory ring (slot = step mod 4: word [32],
-        // residual [32], list entries [32]), copied in with 4-byte cp.async so that no
-        // register waits on a load before its step comes up.
-        auto str_at = [&](int s, int arr) -> unsigned {
-            return str_s + 4u * (unsigned)(((s & 3) * 3 + arr) * 32 + lane);
+        // Streams in the warp's shared-memory ring (slot = step mod 4: words, residuals, list
+        // entries, kStream values each), so that no register waits on a load before its step
+        // comes up.  Copied as the aligned 16-byte vectors that cover the step's values (nine
+        // lanes per array, past the L1; what lies around them is not used), in one instruction
+        // for a step's words and residuals and a later step's list: 4-byte copies, one per lane
+        // and array, went through the L1 and took three.
+        auto str_at = [&](int s, int arr, uint32_t skew) -> unsigned {
+            return str_s + 4u * (unsigned)((s & 3) * 3 * kStream + arr * kStream + (int)skew + lane);
         };
-        auto load_words = [&](int s) {
-            if (s >= s_end) return;
-            const uint32_t inf = __shfl_sync(0xFFFFFFFFu, rec.info, s - wb);
-            const int j0 = __shfl_sync(0xFFFFFFFFu, rec.j0, s - wb);
-            const int hi = (int)(inf & 63u), lo = (int)((inf >> 22) & 31u);
-            if (lane >= lo && lane < hi) {
-                cp4(str_at(s, 0), word + j0 + lane);
-                cp4(str_at(s, 1), a.res + j0 + lane);
-            }
-        };
-        auto load_list = [&](int s) {
-            if (s >= s_end) return;
-            const uint32_t inf = __shfl_sync(0xFFFFFFFFu, rec.info, s - wb);
-            const uint32_t loff = __shfl_sync(0xFFFFFFFFu, rec.list_off, s - wb);
+        auto load_streams = [&](int sw, int sl) {  // words and residuals of sw, list of sl
+            const int j0 = __shfl_sync(0xFFFFFFFFu, rec.j0, sw - wb);
+            const uint32_t loff = __shfl_sync(0xFFFFFFFFu, rec.list_off, sl - wb);
+            const uint32_t inf = __shfl_sync(0xFFFFFFFFu, rec.info, sl - wb);
+            const bool is_list = lane >= 18;
             const int nlist = (int)((inf >> 10) & 63u) + (int)((inf >> 16) & 63u);
-            if (lane < nlist) cp4(str_at(s, 2), list + (size_t)loff + lane);
+            const bool go = is_list ? sl < s_end && str_q < nlist + (int)((inf >> 29) & 3u) : sw < s_end;
+            const uint32_t at = is_list ? loff : (uint32_t)j0;
+            if (go && lane < 27)
+                cp16(str_dst + 4u * (unsigned)(((is_list ? sl : sw) & 3) * 3 * kStream),
+                     str_src + (at & ~3u));
         };
+        auto load_list = [&](int sl) { load_streams(s_end, sl); };
+        auto load_words = [&](int sw) { load_streams(sw, s_end); };
         // stages step s's cold rows (list entries held by its lanes) into pool slot `slot`,
         // and on an item's first step the own row's prev | old regions
         auto stage = [&](int s, int slot) {
             if (s >= s_end) return;
-            int li = 0;
-            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(li) : "r"(str_at(s, 2)));
             const uint32_t inf = __shfl_sync(0xFFFFFFFFu, rec.info, s - wb);
+            int li = 0;
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(li) : "r"(str_at(s, 2, (inf >> 29) & 3u)));
             const int nV = (int)((inf >> 10) & 63u), nR = (int)((inf >> 16) & 63u);
             const unsigned pool = ring_s + 4u * (unsigned)(slot * lp.slot_floats);
             {
@@ -345,8 +355,7 @@ __global__ void __launch_bounds__(lean_max_warps(CM, GK) * kWarp, 1)
         // streams): words and residuals three steps ahead, list entries four ahead, rows
         // one ahead.  At the top of step s every group but the newest is complete: the
         // rows of s (committed at step s - 1), its words (s - 3) and the list of s + 1.
-        load_words(s_begin);
-        load_list(s_begin);
+        load_streams(s_begin, s_begin);
         load_list(s_begin + 1);
         load_list(s_begin + 2);
         load_list(s_begin + 3);
@@ -365,15 +374,14 @@ __global__ void __launch_bounds__(lean_max_warps(CM, GK) * kWarp, 1)
             __syncwarp();
             stage(s + 1, slot ^ 1);
             cp_commit();
-            load_words(s + 3);
-            load_list(s + 4);
+            load_streams(s + 3, s + 4);
             cp_commit();
+            const uint32_t inf = info_of(s);
             uint32_t w0;
             float v0;
-            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w0) : "r"(str_at(s, 0)));
-            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v0) : "r"(str_at(s, 1)));
+            asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w0) : "r"(str_at(s, 0, (inf >> 27) & 3u)));
+            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v0) : "r"(str_at(s, 1, (inf >> 27) & 3u)));
             // ---------------------------------------------------------- compute step s
-            const uint32_t inf = info_of(s);
             const int j0 = __shfl_sync(0xFFFFFFFFu, rec.j0, s - wb);
             const unsigned pool = ring_s + 4u * (unsigned)(slot * lp.slot_floats);
             u64 h[H];
@@ -650,11 +658,11 @@ LeanPlan lean_pass_plan(int CM, bool first, int n, const int64_t *dims_o,
     lp.own_off = kLeanSlots * lp.slot_floats;
     lp.list_off = (lp.own_off + 4 * 2 * CM + 3) / 4 * 4;  // the tensor-core staging follows
     lp.str_off = lp.list_off + stage;  // stream ring: 4 slots x (words, residuals, lists)
-    lp.ring_floats = lp.str_off + 4 * 3 * 32;
+    lp.ring_floats = lp.str_off + 4 * 3 * kStream;
     const size_t kStatic = 2048;  // the kernel's static shared memory (target table) + slack
     const int cspw = std::max(csw[0], csw[1]);
     const size_t warp_bytes =
-        ((((size_t)kLeanSlots * pool_rows * cspw + 8 * CM + 3) / 4 * 4) + stage + 4 * 3 * 32) * 4;
+        ((((size_t)kLeanSlots * pool_rows * cspw + 8 * CM + 3) / 4 * 4) + stage + 4 * 3 * kStream) * 4;
     // as many warps as asked for (default: the most the registers allow) whose rings fit,
     // never more than the kernel's launch bound
     const int max_warps = lean_max_warps(CM, gk);
