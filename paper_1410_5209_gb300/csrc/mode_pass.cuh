@@ -280,6 +280,10 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst)), "l"(src)
                  : "memory");
 }
+__device__ __forceinline__ void cp_async16_l2(void *dst, const void *src) {  // past the L1
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst)), "l"(src)
+                 : "memory");
+}
 template <int BYTES>
 __device__ __forceinline__ void cp_async_small(void *dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(smem_addr(dst)), "l"(src),
@@ -295,6 +299,16 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 __host__ __device__ constexpr size_t align16(size_t b) { return (b + 15) / 16 * 16; }
+// A step's indices and residuals are staged as the aligned 16-byte vectors that cover them:
+// 32 values from anywhere in a vector of `per` values, and where the step's first one lies.
+__host__ __device__ constexpr int window(int per) { return 32 / per * per + per; }
+// NO > 2 only: the vectors' bookkeeping costs three-way passes more than the narrower copies
+// (C = 4: 0.70 against 0.66 ms).
+template <class T, int NO>
+__host__ __device__ constexpr int window_skew(int j0) {
+    return NO > 2 ? j0 & (16 / (int)sizeof(T) - 1) : 0;
+}
+constexpr int kIdxWin = window(4);
 __host__ __device__ constexpr int odd_up(int v) { return v | 1; }
 
 struct Step {  // nnz < 2^31, so entry positions fit in 32 bits
@@ -350,9 +364,9 @@ struct PipeGeo {
         return align16(slot_elems(no > 0 ? no : 1, n_lo) * sizeof(T));
     }
     static __host__ __device__ size_t ridx_bytes(int no) {
-        return align16((size_t)(no > 0 ? no : 1) * 32 * 4);
+        return align16((size_t)(no > 0 ? no : 1) * kIdxWin * 4);
     }
-    static constexpr size_t RV_BYTES = align16(32 * sizeof(T));
+    static constexpr size_t RV_BYTES = align16(window(V) * sizeof(T));
     static constexpr size_t OWN_BYTES = align16(2 * CM * sizeof(T));
     static __host__ __device__ size_t heads_bytes(int no) {
         return align16((size_t)(no > 0 ? no : 1) * 4);
@@ -422,12 +436,34 @@ __device__ __forceinline__ void issue_idx(const Step &s, int32_t *ridx, T *rv, T
                                           const tf_item *items, const T *Zn, const int32_t *rank_n,
                                           int own_off, int own_len, int lane) {
     if (!(s.flags & 1)) return;
-    const int j = s.j0 + lane;
-    if (j < s.jend) {
-        const int no = om.count();
+    if constexpr (NO > 2) {
+        constexpr int V = 16 / (int)sizeof(T);
+        // a 16-byte copy per lane, in two rounds, instead of a 4-byte one per lane and array;
+        // the arrays end in padding
+        const int si = window_skew<int32_t, NO>(s.j0), sr = window_skew<T, NO>(s.j0);
+        constexpr int VI = kIdxWin / 4, VR = window(V) / V, ALL = NO * VI + VR;
+        const int n = min(s.jend - s.j0, kWarp);
+#pragma unroll
+        for (int q0 = 0; q0 < ALL; q0 += kWarp) {
+            const int q = q0 + lane, t = q / VI, v = q - t * VI;
+            if (t < NO) {
+                const int32_t *src = om.oidx[0];
+#pragma unroll
+                for (int k = 1; k < NO; ++k) src = t == k ? om.oidx[k] : src;
+                if (4 * v < n + si) cp_async16_l2(ridx + t * kIdxWin + 4 * v, src + (s.j0 - si) + 4 * v);
+            } else {
+                const int w = q - NO * VI;
+                if (w < VR && V * w < n + sr) cp_async16_l2(rv + V * w, res + (s.j0 - sr) + V * w);
+            }
+        }
+    } else {
+        const int j = s.j0 + lane;
+        if (j < s.jend) {
+            const int no = om.count();
 #pragma unroll(NO > 0 ? NO : 1)
-        for (int t = 0; t < no; ++t) cp_async_small<4>(ridx + t * 32 + lane, om.oidx[t] + j);
-        cp_async_small<sizeof(T)>(rv + lane, res + j);
+            for (int t = 0; t < no; ++t) cp_async_small<4>(ridx + t * kIdxWin + lane, om.oidx[t] + j);
+            cp_async_small<sizeof(T)>(rv + lane, res + j);
+        }
     }
     if ((s.flags & 2) && lane < own_len) {
         const int64_t row = rank_n[items[s.it].row];
@@ -450,7 +486,7 @@ __device__ __forceinline__ void issue_rows(const Step &s, T *rows, uint32_t *hea
     const int part = lane & (G::NV - 1), rsub = lane / G::NV;
 #pragma unroll(NO > 0 ? NO : 1)
     for (int t = 0; t < no; ++t) {
-        const int32_t *ri = ridx + t * 32;
+        const int32_t *ri = ridx + t * kIdxWin + window_skew<int32_t, NO>(s.j0);
         const int mine = ri[lane], before = lane > 0 ? ri[lane - 1] : -1;
         const uint32_t hm =
             __ballot_sync(0xFFFFFFFFu, lane < nvalid && (lane == 0 || mine != before));
@@ -463,8 +499,15 @@ __device__ __forceinline__ void issue_rows(const Step &s, T *rows, uint32_t *hea
 #pragma unroll
         for (int k = 0; k < G::NV; ++k) {
             const int row = k * RPR + rsub;
-            if ((hm >> row) & 1u)
-                cp_async16(dst + k * RPR * rs, Z + (int64_t)ri[row] * G::W);
+            if ((hm >> row) & 1u) {
+                // through the L1, which holds hot rows; four other modes' rows leave it no
+                // room for that (five-way, 2e7 entries: last mode 2.80 ms, 2.52 past it; 256
+                // small three-way tensors the other way, 0.67 and 0.74)
+                if (NO > 2)
+                    cp_async16_l2(dst + k * RPR * rs, Z + (int64_t)ri[row] * G::W);
+                else
+                    cp_async16(dst + k * RPR * rs, Z + (int64_t)ri[row] * G::W);
+            }
         }
     }
 }
@@ -750,7 +793,7 @@ struct PassConsumer {
         }
         T h[CM], po = T(0), pp = T(0);
         entry_products<T, CM, NO, FIRST>(rowp, sm.own, no, n_lo, a.C, a.Cq, h, po, pp);
-        T v = sm.rv(is)[lane];
+        T v = sm.rv(is)[window_skew<T, NO>(st.j0) + lane];
         if (FIRST) {
             v = v - pp + po;
             a.res[j] = v;
@@ -1165,7 +1208,7 @@ struct ResConsumer {
             for (int c = 0; c < CM; ++c)
                 if (c < a.Cq) p += q[c];
         }
-        const T r = sm.rv(is)[lane] - p;
+        const T r = sm.rv(is)[window_skew<T, NO>(st.j0) + lane] - p;
         if (a.what == 0)
             acc += (double)r * (double)r;
         else if (a.what == 1)
