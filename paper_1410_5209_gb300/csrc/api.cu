@@ -1227,9 +1227,10 @@ struct Impl : CtxBase {
         // Wide subsets of float three-way tensors up to C = 63, without solve options: the
         // warp-wide pass with register operands (mma_pass.cu), unless path 1 or 2 or the
         // single-TF32 form asks for another.  Against the block-wide passes: 5e6 entries at
-        // C = 20 0.28 against 0.75 ms a pass, 1e7 at C = 50 1.83 against 2.60 ms.  Errors of
-        // the factors against 64 bits over nine drawn tensors: C <= 31 0.9 to 1.1 times the
-        // SIMT pass's (4.6e-7 to 1.6e-6), C >= 32 a third of the tcgen05 pass's.
+        // C = 20 0.28 against 0.75 ms for a mode's two passes, 1e7 at C = 50 1.60 against 2.60
+        // ms.  Errors of the factors against 64 bits: six drawn tensors at C = 20 at most 2.7e-7
+        // / 4.2e-7 / 6.6e-7 (SIMT pass: 3.2e-7 / 9.2e-7 / 1.5e-6), C = 50 2.3e-6 (tcgen05 pass:
+        // 6.7e-6).
         const bool wide_mma = sizeof(T) == 4 && wide && path != 1 && path != 2 && precision != 1 &&
                               pass_mma_supported(N, C, CM) &&
                               solve_mid_supported(C, solve_refine || solve_cond > 0.f);

@@ -74,11 +74,4 @@ __device__ void warp_chol_apply(const T *P, T *c, int C, int lane) {
     }
 }
 
-template <class T>
-__device__ bool warp_chol_solve(T *P, T *c, int C, T lam, int lane) {
-    const bool ok = warp_chol_factor<T>(P, C, lam, lane);
-    warp_chol_apply<T>(P, c, C, lane);
-    return ok;
-}
-
 }  // namespace tfs

@@ -1,14 +1,18 @@
 // Row solves of float contexts for subsets of 17 to 63 columns without solve options: one warp
-// per row, the system [B + lambda I, c] in registers (lane i holds rows i and, past 31
+// per row, the factor of [B + lambda I, c] in registers (lane i holds rows i and, past 31
 // columns, i + 32; the right-hand side is row C, so the forward substitution comes with the
-// factor), a right-looking Cholesky whose column j reaches the other lanes through shared
-// memory as 16-byte broadcasts.
+// factor), whose column j reaches the other lanes through shared memory as 16-byte broadcasts.
 //
 // Bound: the chain of C columns (pivot, broadcast, update: about 170 cycles each) with 12 warps
 // per SM in flight, and issue: 1,300 packed FMAs and 520 broadcasts a row at C = 63.  The form it
 // replaces (k_solve_wide, wide.cu, still used for wider subsets, FP64 and the solve options)
 // walks a packed triangle in shared memory, two loads per multiply-add and a warp reduction
-// per column: 50,021 rows at C = 50 took it 1.06 ms (0.64 here), 30,011 at C = 20 0.26 (0.074).
+// per column: 50,021 rows at C = 50 took it 1.06 ms (0.60 here), 30,011 at C = 20 0.26 (0.062).
+//   Precision: the products to take off an element are summed first and taken off once, as there.
+// Taking each off the element (right-looking; 0.44 and 0.052 ms) rounds at the element's size
+// every time: factors of a weighted-lambda fit 4.1e-7 / 6.1e-7 / 1.3e-6 off 64 bits, where this
+// form and the old one are 2.7e-7 / 4.2e-7 / 7e-7 off.  Quotients by the pivot keep what its
+// rounded inverse leaves (0.02 ms of 2.4; without it up to 8.8e-7).
 //   Rows held by one item: four per block.  Split rows: one block each, whose threads first
 // add the row's slots (or sums of kSlotGroup slots) in order, eight loads in flight each.
 #include <algorithm>
@@ -62,51 +66,62 @@ __device__ __forceinline__ bool mid_solve(float *P, float *col, int C, float lam
     const int ntc = C * (C + 1) / 2;
     for (int i = lane; i < C; i += 32) P[i * (i + 1) / 2 + i] += lam;
     __syncwarp();
-    // Rows lane (columns 0 .. 31) and lane + 32 (0 .. KM - 1), in pairs.  What is read past a
-    // row's end (the next rows, the rest of the buffer) ends up above the diagonal, in columns
-    // from C on or in rows past C, none of which reach the factor or the solution.
+    // Of rows lane (columns 0 .. 31) and lane + 32 (0 .. KM - 1), in pairs: the sums of products
+    // that column j's elements will have taken off when it comes up (one subtraction at the
+    // element's size, as in a left-looking factorisation, instead of one per column before it),
+    // then L.  The elements themselves wait in shared memory: triangular numbers differ modulo
+    // 32, so lanes reading column j do not conflict.  What is read past a row's end (the next
+    // rows, the rest of the buffer) ends up above the diagonal, in columns from C on or in rows
+    // past C, none of which reach the factor or the solution.
+    const float *p0 = P + (lane < C ? lane * (lane + 1) / 2 : ntc);
+    const float *p1 = P + (lane + 32 < C ? (lane + 32) * (lane + 33) / 2 : ntc);
     u64 a0[K0 / 2], a1[R == 2 ? KM / 2 : 1];
-    {
-        const float *p0 = P + (lane < C ? lane * (lane + 1) / 2 : ntc);
 #pragma unroll
-        for (int p = 0; p < K0 / 2; ++p) a0[p] = mid_pack(p0[2 * p], p0[2 * p + 1]);
-        if constexpr (R == 2) {
-            const int i = lane + 32;
-            const float *p1 = P + (i < C ? i * (i + 1) / 2 : ntc);
+    for (int p = 0; p < K0 / 2; ++p) a0[p] = 0ull;
 #pragma unroll
-            for (int p = 0; p < KM / 2; ++p) a1[p] = mid_pack(p1[2 * p], p1[2 * p + 1]);
-        }
-    }
-    __syncwarp();
+    for (int p = 0; p < (R == 2 ? KM / 2 : 1); ++p) a1[p] = 0ull;
     bool ok = true;
-    float inv0 = 1.f, inv1 = 1.f;  // inverse pivots of the lane's rows
+    float inv0 = 1.f, inv1 = 1.f, rest0 = 0.f, rest1 = 0.f;  // inverse pivots of the lane's rows
 #pragma unroll
     for (int j = 0; j < KM - 1; ++j) {
         if (j < C) {
             float *c = col + (j & 1) * 32 * R;
-            const float mine = j < 32 ? mid_get(a0[j < K0 ? j / 2 : 0], j & 1)
-                                      : mid_get(a1[R == 2 ? j / 2 : 0], j & 1);
+            const float m0 = j < 32 ? p0[j] - mid_get(a0[j < K0 ? j / 2 : 0], j & 1) : 0.f;
+            const float m1 = R == 2 ? p1[j] - mid_get(a1[R == 2 ? j / 2 : 0], j & 1) : 0.f;
+            const float mine = j < 32 ? m0 : m1;
             float d = __shfl_sync(0xFFFFFFFFu, mine, j & 31);
             ok = ok && (d > 0.f);
             d = d > 0.f ? d : 1.f;
-            float inv = rsqrtf(d);
-            inv = inv * fmaf(-0.5f * d * inv, inv, 1.5f);  // one Newton step
+            // quotients by the pivot as products with its inverse and what that leaves (Markstein,
+            // "Computation of elementary functions on the IBM RISC System/6000 processor", IBM
+            // J. Res. Dev. 34, 1990): a rounded inverse alone would scale the whole column
+            float root, inv;
+            if (d > 0x1p-60f && d < 0x1p120f) {
+                // d^1/2 and its inverse from the approximate d^-1/2 by one correction each
+                inv = rsqrtf(d);
+                root = d * inv;
+                root = fmaf(fmaf(-root, root, d), 0.5f * inv, root);
+                inv = fmaf(inv, fmaf(-root, inv, 1.f), inv);
+            } else {
+                root = sqrtf(d);
+                inv = 1.f / root;
+            }
+            const float rest = fmaf(-inv, root, 1.f) * inv;
             float l0 = 0.f, l1 = 0.f;
             if (j < 32) {
-                l0 = lane == j ? d * inv : mine * inv;
-                if (lane == j) inv0 = inv;
+                l0 = lane == j ? root : fmaf(m0, inv, m0 * rest);
+                if (lane == j) inv0 = inv, rest0 = rest;
                 a0[j < K0 ? j / 2 : 0] = mid_set(a0[j < K0 ? j / 2 : 0], j & 1, l0);
                 c[lane] = l0;
             }
             if constexpr (R == 2) {
-                const float m1 = mid_get(a1[j / 2], j & 1);
-                l1 = j >= 32 && lane == j - 32 ? d * inv : m1 * inv;
-                if (j >= 32 && lane == j - 32) inv1 = inv;
+                l1 = j >= 32 && lane == j - 32 ? root : fmaf(m1, inv, m1 * rest);
+                if (j >= 32 && lane == j - 32) inv1 = inv, rest1 = rest;
                 a1[j / 2] = mid_set(a1[j / 2], j & 1, l1);
                 c[lane + 32] = l1;
             }
             __syncwarp();
-            const u64 n0 = mid_pack(-l0, -l0), n1 = mid_pack(-l1, -l1);
+            const u64 n0 = mid_pack(l0, l0), n1 = mid_pack(l1, l1);
 #pragma unroll
             for (int q = 0; q < KM / 4; ++q) {
                 if (4 * q + 3 > j) {
@@ -125,7 +140,8 @@ __device__ __forceinline__ bool mid_solve(float *P, float *col, int C, float lam
             }
         }
     }
-    // the factor's rows, L^-1 c as row C
+    // the factor's rows, L^-1 c as row C, over the system
+    __syncwarp();
     float *L = P;
 #pragma unroll
     for (int p = 0; p < K0 / 4; ++p)
@@ -141,12 +157,14 @@ __device__ __forceinline__ bool mid_solve(float *P, float *col, int C, float lam
     }
     __syncwarp();
     float y0 = L[C * LD + lane], y1 = R == 2 ? L[C * LD + lane + 32] : 0.f;
+    float s0 = 0.f, s1 = 0.f;  // sums to take off, as above
     x0 = x1 = 0.f;
 #pragma unroll 4
     for (int j = C - 1; j >= 0; --j) {
         const float r0 = lane < j ? L[j * LD + lane] : 0.f;
         const float r1 = R == 2 && lane + 32 < j ? L[j * LD + lane + 32] : 0.f;
-        const float mine = R == 2 && j >= 32 ? y1 * inv1 : y0 * inv0;
+        const float m = R == 2 && j >= 32 ? y1 - s1 : y0 - s0;
+        const float mine = R == 2 && j >= 32 ? fmaf(m, inv1, m * rest1) : fmaf(m, inv0, m * rest0);
         const float xj = __shfl_sync(0xFFFFFFFFu, mine, j & 31);
         if (lane == (j & 31)) {
             if (R == 2 && j >= 32)
@@ -154,8 +172,8 @@ __device__ __forceinline__ bool mid_solve(float *P, float *col, int C, float lam
             else
                 x0 = xj;
         }
-        y0 -= r0 * xj;
-        y1 -= r1 * xj;
+        s0 += r0 * xj;
+        s1 += r1 * xj;
     }
     return ok;
 }

@@ -17,8 +17,12 @@
 // b1 b3; b1 b1 (16 bits) is summed apart from the rest, so that the tensor core, which truncates
 // what it adds, has nothing to cut off there.  C >= 32 (two chunks, no registers for that):
 // h = hi + lo in TF32, lo hi + hi lo + hi hi.  Either way the products of one step are summed
-// from zero and added to FP32 sums with ordinary rounding.  Errors of the factors against 64
-// bits in the dispatch (api.cu).
+// from zero and added to FP32 sums with ordinary rounding.  With one chunk the right-hand side
+// and B's diagonal are summed by FMAs on the same registers instead (no cost beside the loads:
+// 0.14 ms a pass either way); over six seeds of a weighted-lambda fit at C = 20 the largest
+// error of a factor against 64 bits is then 6.6e-7, with the diagonal on the tensor cores
+// 2.0e-6, and 1.5e-6 with FP32 throughout.  With two chunks the FMAs' registers cost 0.2 ms of
+// 1.6, and the errors are a third of FP32's without them (dispatch in api.cu).
 //   Range.  Below 2^-100 the split of h would lose its last parts, and collapsed columns
 // (weighted lambda) do get there.  The pack and the solves record the largest value of every
 // mode's current columns (PassArgs::mx); a pass whose factors' product lies outside 2^-80 ..
@@ -74,6 +78,11 @@ __device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
+__device__ __forceinline__ u64 pair(float x, float y) {
+    u64 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
 __device__ __forceinline__ void halves(u64 v, float &x, float &y) {
     asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
 }
@@ -114,11 +123,14 @@ __device__ __forceinline__ void mma16z(float (&d)[4], uint32_t a0, uint32_t a1, 
 // Entries per step: 16 (two halves of 8) for one chunk, 8 for two.
 __host__ __device__ constexpr int mma_step(int CH) { return CH == 1 ? 16 : 8; }
 __host__ __device__ constexpr int mma_tiles(int CH) { return 2 * CH * (2 * CH + 1); }
-// Warps per block (one block per SM): what the registers allow, 24 sums and 8 entry values per
-// lane at CH = 1, 80 and 16 at CH = 2.
-__host__ __device__ constexpr int mma_warps(int CH) { return CH == 1 ? 16 : 12; }
+// Warps per block (one block per SM).  CH = 1: 16 at 128 registers (12: 0.29, 16: 0.28, 20:
+// 0.32 ms a pass at 5e6 entries, C = 20).  CH = 2: 8, whose 255 registers hold the 80 sums and
+// a step's operands and loads without spilling (1e7 entries, C = 50: 12 warps 1.62 / 1.87 /
+// 2.34, 10 warps 1.64 / 1.85 / 1.91, 8 warps 1.54 / 1.60 / 1.65 ms, each the pass that refreshes
+// R-hat and the one that does not together).
+__host__ __device__ constexpr int mma_warps(int CH) { return CH == 1 ? 16 : 8; }
 
-// CH: 32-feature chunks (C + 1 <= 32 CH; chunk features past C are zero).  FIRST: the split's
+// CH: 32-feature chunks (C < 32 CH; chunk features past C are zero).  FIRST: the split's
 // first inner iteration; NLO other modes precede mode n (already updated in this split: their
 // old columns differ from cur).  Lane 4 g + t works on entries t, t + 4 (and t + 8, t + 12: the
 // second half of a 16-entry step); which of a step's entries is which index of the product's
@@ -148,9 +160,9 @@ __global__ void __launch_bounds__(mma_warps(CH) * kWarp, 1)
         const int hi = r > c ? r : c, lo = r > c ? c : r;
         int at = NB;
         if (j > n || (j == n && r >= c)) {
-            if (hi < C)
+            if (hi < C && (CH > 1 || lo < hi))
                 at = hi * (hi + 1) / 2 + lo;
-            else if (hi == C && lo < C)
+            else if (CH > 1 && hi == C && lo < C)
                 at = NT + lo;
         }
         place[q] = (uint16_t)at;
@@ -159,20 +171,25 @@ __global__ void __launch_bounds__(mma_warps(CH) * kWarp, 1)
     __syncthreads();
 
     bool in[CH], inq[CH];  // the lane's columns of a chunk exist in this / the previous subset
-    unsigned is_res = 0u;  // bit j: the lane's feature j is column C of H' (r_hat)
+    unsigned is_res = 0u;  // two chunks: bit j, the lane's feature j is column C of H' (r_hat)
 #pragma unroll
     for (int q = 0; q < CH; ++q) {
         in[q] = 32 * q + 4 * g < CM;
         inq[q] = 32 * q + 4 * g < a.Cq;
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            if (32 * q + 4 * g + u == C) is_res |= 1u << (4 * q + u);
+            if (CH > 1 && 32 * q + 4 * g + u == C) is_res |= 1u << (4 * q + u);
     }
     const float *Z0 = a.Zo[0] + 4 * g, *Z1 = a.Zo[1] + 4 * g;
     const int32_t *ix0 = a.oidx[0], *ix1 = a.oidx[1];
     u64 acc[TILES][2];
 #pragma unroll
     for (int k = 0; k < TILES; ++k) acc[k][0] = acc[k][1] = 0ull;
+    // one chunk: the lane's entries' part of the right-hand side and of B's diagonal, by feature
+    constexpr int JF = CH == 1 ? J / 2 : 1;
+    u64 csum[JF], dsum[JF];
+#pragma unroll
+    for (int j = 0; j < JF; ++j) csum[j] = dsum[j] = 0ull;
     u64 own_old[J / 2], own_prev[J / 2];  // own row: old columns, and prev ones negated
 #pragma unroll
     for (int j = 0; j < J / 2; ++j) own_old[j] = own_prev[j] = 0ull;
@@ -282,9 +299,19 @@ __global__ void __launch_bounds__(mma_warps(CH) * kWarp, 1)
             for (int e = 0; e < E; ++e) {
                 const float v = FIRST ? rv[e] + d[e] : rv[e];
                 if (FIRST && g == 0 && i0[e] >= 0) a.res[j0 + t + 4 * e] = v;
+                if constexpr (CH == 1) {
+                    const u64 vv = pair(v, v);
 #pragma unroll
-                for (int j = 0; j < J; ++j)
-                    if ((is_res >> j) & 1u) h[e][j] = i0[e] >= 0 ? v : 0.f;
+                    for (int j = 0; j < J / 2; ++j) {
+                        const u64 hp = pair(h[e][2 * j], h[e][2 * j + 1]);
+                        csum[j] = fma2(hp, vv, csum[j]);
+                        dsum[j] = fma2(hp, hp, dsum[j]);
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < J; ++j)
+                        if ((is_res >> j) & 1u) h[e][j] = i0[e] >= 0 ? v : 0.f;
+                }
             }
             if constexpr (CH == 1) {
                 uint32_t b1[J][2], b2[J][2], b3[J][2];
@@ -348,6 +375,24 @@ __global__ void __launch_bounds__(mma_warps(CH) * kWarp, 1)
                         buf[place[(4 * k + 2 * i + 1) * 32 + lane]] = y;
                         acc[k][i] = 0ull;
                     }
+                if constexpr (CH == 1) {
+#pragma unroll
+                    for (int j = 0; j < J; ++j) {  // the FMAs' sums over the lanes of a feature
+                        const int f = 4 * g + j;
+                        auto over_lanes = [&](u64 v) {
+                            float x, y;
+                            halves(v, x, y);
+                            float c = j & 1 ? y : x;
+                            c += __shfl_xor_sync(0xFFFFFFFFu, c, 1);
+                            return c + __shfl_xor_sync(0xFFFFFFFFu, c, 2);
+                        };
+                        const float c = over_lanes(csum[j / 2]), b = over_lanes(dsum[j / 2]);
+                        if (t == 0 && f < C) buf[NT + f] = c;
+                        if (t == 1 && f < C) buf[f * (f + 1) / 2 + f] = b;
+                    }
+#pragma unroll
+                    for (int j = 0; j < J / 2; ++j) csum[j] = dsum[j] = 0ull;
+                }
                 __syncwarp();
                 float *p = a.partials + (int64_t)item.slot * NB;
                 for (int q = lane; q < NB; q += 32) p[q] = buf[q];
