@@ -292,7 +292,8 @@ tf_status tf_get_residual(tf_ctx *ctx, void *host_r);
  * counters[3] = work items of all modes, counters[4] = rows split across bins,
  * counters[5] = bins P of the schedule, counters[6] = kernels launched by the last
  * tf_loss, counters[7] = mode-pass data paths the last sweep used (bit 0: SIMT pass,
- * bit 1: TMA gather pass, bit 2: tensor-core Gram pass of wide subsets; 0 = no sweep). */
+ * bit 1: TMA gather pass, bit 2: tensor-core Gram pass of wide subsets, with bit 0 where a
+ * SIMT kernel stands behind it; 0 = no sweep). */
 tf_status tf_get_counters(tf_ctx *ctx, int64_t counters[8]);
 
 /* Re-plans the row schedule of every mode (policy, P bins; P = 0 picks the default
@@ -304,9 +305,12 @@ tf_status tf_set_schedule(tf_ctx *ctx, tf_sched_policy policy, int P);
 
 /* Data path of the mode pass: 0 = automatic (C <= 16: for float three-way tensors and
  * C <= 12 the lean pass (hot slice rows resident in shared memory, packed two-wide FP32
- * Gram), else the cp.async SIMT pass; 16 < C < 128: for float contexts the Gram on the
- * tensor cores (tcgen05, three TF32 products per term, FP32 accumulation) for C >= 32,
- * where it measures faster, SIMT FMAs below and for double), 1 = the cp.async SIMT pass
+ * Gram), else the cp.async SIMT pass; float three-way 16 < C < 64 without solve options
+ * and unless tf_set_precision(1): the Gram on the tensor cores from registers (bfloat16 or TF32
+ * splits at FP32 level; factors whose products leave the splits' range take the kernels
+ * named next); other 16 < C < 128: for float contexts the Gram on the tensor cores
+ * (tcgen05, three TF32 products per term, FP32 accumulation) for C >= 32, where it
+ * measures faster, SIMT FMAs below and for double), 1 = the cp.async SIMT pass
  * and the SIMT wide Gram everywhere, 2 = the TMA tile::gather4 pass with its shared-memory row cache for
  * C <= 10 (float, N = 3; TF_EINVAL from the next sweep where it does not apply) and the
  * tensor-core Gram for every wide C, 3 = the lean pass (TF_EINVAL from the next sweep
@@ -368,10 +372,10 @@ tf_status tf_device_peaks(double *fp32_tflops, double *fp32x2_tflops, double *sm
 typedef enum {
     TF_KIND_PACK = 0,      /* slice packing of a split (Theorem 3's C resident columns) */
     TF_KIND_MODE_PASS = 1, /* fused R-hat / Gram / rhs pass over one mode (Eq. 4)        */
-    TF_KIND_COMBINE = 2,   /* sum of split rows' partial Gram/rhs + Cholesky solve      */
+    TF_KIND_COMBINE = 2,   /* wide C: sums of split rows' partial Gram/rhs (and solves)  */
     TF_KIND_LOSS = 3,      /* loss / residual reductions (Eq. 1)                        */
     TF_KIND_OTHER = 4,     /* residual rebuilds and flushes                             */
-    TF_KIND_SOLVE = 5,     /* Cholesky solves of the rows held by one item (Sec. 3.1)   */
+    TF_KIND_SOLVE = 5,     /* Cholesky row solves, split rows' sums included (Sec. 3.1)  */
     TF_KIND_COUNT = 6
 } tf_kernel_kind;
 

@@ -1,5 +1,6 @@
-"""The pass over four- and five-way tensors stages a step's indices and residuals as the 16-byte
-vectors that cover them: items that start and end anywhere in a vector, and at the arrays' end."""
+"""The pass over five-way tensors stages a step's indices and residuals as the 16-byte vectors
+that cover them: items that start and end anywhere in a vector, and at the arrays' end.  Four-way
+tensors run the generic form, which copies value by value."""
 import numpy as np
 import pytest
 
