@@ -38,7 +38,7 @@ WORKLOAD = dict(workload="skewed_3way_1e8", dims=[100_000, 100_000, 1_000], nnz=
 # reports traffic as null once the sources differ or the entry count is not 1e8.
 NCU_TRAFFIC = 1.689e9
 NCU_TRAFFIC_NNZ = 100_000_000
-NCU_SOURCE_HASH = "bf274e857376da3a"
+NCU_SOURCE_HASH = "44bc8037a965156d"
 
 
 # Utilisation of the L1 data pipe (shared-memory and L1 wavefronts) of the mode pass in the

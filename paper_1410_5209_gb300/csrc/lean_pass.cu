@@ -83,6 +83,9 @@ __device__ __forceinline__ u64 lds1(unsigned a) {
     asm volatile("ld.shared.b64 %0, [%1];" : "=l"(x) : "r"(a));
     return x;
 }
+// past the L1: a row staged in the pool is not read again from there before the L1, which the
+// caches and rings leave little of, has dropped it (1e8 entries, C = 10: sweep and loss 60.7 ms
+// through it, 58.1 past it)
 __device__ __forceinline__ void cp16(unsigned dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
 }
@@ -286,7 +289,8 @@ __global__ void __launch_bounds__(lean_max_warps(CM, GK) * kWarp, 1)
         // comes up.  Copied as the aligned 16-byte vectors that cover the step's values (nine
         // lanes per array, past the L1; what lies around them is not used), in one instruction
         // for a step's words and residuals and a later step's list: 4-byte copies, one per lane
-        // and array, went through the L1 and took three.
+        // and array, went through the L1 and took three (1e8
+        // entries, C = 10: sweep and loss 58.1 ms with those, 53.9 now).
         auto str_at = [&](int s, int arr, uint32_t skew) -> unsigned {
             return str_s + 4u * (unsigned)((s & 3) * 3 * kStream + arr * kStream + (int)skew + lane);
         };

@@ -124,7 +124,7 @@ __device__ __forceinline__ void mma16z(float (&d)[4], uint32_t a0, uint32_t a1, 
 __host__ __device__ constexpr int mma_step(int CH) { return CH == 1 ? 16 : 8; }
 __host__ __device__ constexpr int mma_tiles(int CH) { return 2 * CH * (2 * CH + 1); }
 // Warps per block (one block per SM).  CH = 1: 16 at 128 registers (12: 0.29, 16: 0.28, 20:
-// 0.32 ms a pass at 5e6 entries, C = 20).  CH = 2: 8, whose 255 registers hold the 80 sums and
+// 0.32 ms for a mode's two passes at 5e6 entries, C = 20).  CH = 2: 8, whose 255 registers hold the 80 sums and
 // a step's operands and loads without spilling (1e7 entries, C = 50: 12 warps 1.62 / 1.87 /
 // 2.34, 10 warps 1.64 / 1.85 / 1.91, 8 warps 1.54 / 1.60 / 1.65 ms, each the pass that refreshes
 // R-hat and the one that does not together).
