@@ -238,9 +238,12 @@ tf_status plan_mode(const int64_t *off, int64_t I, int P, int64_t cap, tf_sched_
     const int64_t nnz = I > 0 ? off[I] : 0;
     if (cap == 0) cap = std::max<int64_t>(1, (nnz + P - 1) / P);
 
-    for (int64_t i = 0; i < I; ++i)
-        if (off[i + 1] - off[i] > INT32_MAX && !(policy == TF_SCHED_LPT && cap <= INT32_MAX))
-            return TF_EINVAL;
+    // an item's length is 32 bits: a whole row's, or that of a long row's chunks
+    for (int64_t i = 0; i < I; ++i) {
+        const int64_t len = off[i + 1] - off[i];
+        const int64_t chunks = policy == TF_SCHED_LPT && len > cap ? (len + cap - 1) / cap : 1;
+        if (len > INT32_MAX && (len + chunks - 1) / chunks > INT32_MAX) return TF_EINVAL;
+    }
     if (policy == TF_SCHED_LPT) {
         // jobs: whole rows, or near-equal chunks of rows longer than cap; one slot each, in
         // row order, so a job's number is its slot
