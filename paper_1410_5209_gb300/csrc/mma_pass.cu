@@ -30,6 +30,7 @@
 // opposite gate (one of the two returns at once).
 #include <algorithm>
 
+#include "entry_steps.h"
 #include "sweep.cuh"
 
 namespace tfs {
@@ -203,7 +204,7 @@ __global__ void __launch_bounds__(mma_warps(CH) * kWarp, 1)
         const int64_t it_end = a.bin_ptr[tk + 1];
         if (it >= it_end) continue;
         tf_item item = a.items[it];
-        int j0 = (int)item.begin, jend = (int)(item.begin + item.len);  // nnz < 2^31
+        int j0 = (int)item.begin, jend = (int)(item.begin + item.len);
         bool fresh = true;
         // indices and residuals of the lane's entries (t, t + 4, ...), one step ahead
         int32_t i0[E], i1[E];
@@ -211,10 +212,10 @@ __global__ void __launch_bounds__(mma_warps(CH) * kWarp, 1)
         auto load_entries = [&](int j, int end, int32_t (&x0)[E], int32_t (&x1)[E], float (&r)[E]) {
 #pragma unroll
             for (int e = 0; e < E; ++e) {
-                const int at = j + t + 4 * e;
                 x0[e] = x1[e] = -1;
                 r[e] = 0.f;
-                if (at < end) {
+                if (has_entry(j, t + 4 * e, end)) {
+                    const int at = j + (t + 4 * e);
                     x0[e] = ix0[at];
                     x1[e] = ix1[at];
                     r[e] = a.res[at];
@@ -239,10 +240,10 @@ __global__ void __launch_bounds__(mma_warps(CH) * kWarp, 1)
                 }
             }
             // the next step's entries
-            const bool last = j0 + STEP >= jend;
-            tf_item next = item;
-            int nj = j0 + STEP, nend = jend;
+            const bool last = last_step(j0, STEP, jend);
             const bool more = !last || it + 1 < it_end;
+            tf_item next = item;
+            int nj = last ? jend : j0 + STEP, nend = jend;  // none after the bin's last step
             if (last && more) {
                 next = a.items[it + 1];
                 nj = (int)next.begin;
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(mma_warps(CH) * kWarp, 1)
             }
             int32_t n0[E], n1[E];
             float nr[E];
-            load_entries(nj, more ? nend : 0, n0, n1, nr);
+            load_entries(nj, nend, n0, n1, nr);
 
             // products of this step
             float h[E][J], d[E];

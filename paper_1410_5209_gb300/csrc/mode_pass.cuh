@@ -21,6 +21,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "entry_steps.h"
 #include "sweep.cuh"
 
 namespace tfs {
@@ -311,35 +312,13 @@ __host__ __device__ constexpr int window_skew(int j0) {
 constexpr int kIdxWin = window(4);
 __host__ __device__ constexpr int odd_up(int v) { return v | 1; }
 
-struct Step {  // nnz < 2^31, so entry positions fit in 32 bits
-    int32_t j0, jend;
-    int32_t it;
-    int32_t flags;  // 1 valid, 2 first step of its item, 4 last step of its item
-};
-
 __device__ __forceinline__ Step step_at_item(const tf_item *items, int64_t it, int64_t it_end) {
-    Step s;
-    s.it = (int32_t)it;
-    if (it >= it_end) {
-        s.j0 = s.jend = 0;
-        s.flags = 0;
-        return s;
-    }
-    const tf_item x = items[it];
-    s.j0 = (int32_t)x.begin;
-    s.jend = (int32_t)(x.begin + x.len);
-    s.flags = 1 | 2 | ((x.len <= kWarp) ? 4 : 0);
-    return s;
+    return it < it_end ? first_step(items[it], it) : no_step(it);
 }
 
 __device__ __forceinline__ Step step_next(const Step &s, const tf_item *items, int64_t it_end) {
     if (!(s.flags & 1)) return s;
-    if (s.j0 + kWarp < s.jend) {
-        Step n = s;
-        n.j0 += kWarp;
-        n.flags = 1 | ((n.j0 + kWarp >= n.jend) ? 4 : 0);
-        return n;
-    }
+    if (!(s.flags & 4)) return step_on(s);
     return step_at_item(items, (int64_t)s.it + 1, it_end);
 }
 
@@ -457,8 +436,8 @@ __device__ __forceinline__ void issue_idx(const Step &s, int32_t *ridx, T *rv, T
             }
         }
     } else {
-        const int j = s.j0 + lane;
-        if (j < s.jend) {
+        if (has_entry(s.j0, lane, s.jend)) {
+            const int j = s.j0 + lane;
             const int no = om.count();
 #pragma unroll(NO > 0 ? NO : 1)
             for (int t = 0; t < no; ++t) cp_async_small<4>(ridx + t * kIdxWin + lane, om.oidx[t] + j);
@@ -776,8 +755,8 @@ struct PassConsumer {
         }
     }
     __device__ __forceinline__ void entry(const SM &sm, const Step &st, int rs, int is, int lane) {
+        if (!has_entry(st.j0, lane, st.jend)) return;
         const int j = st.j0 + lane;
-        if (j >= st.jend) return;
         const T *slot = sm.rows(rs);
         const uint32_t *hd = sm.heads(rs);
         constexpr int NP = NO > 0 ? NO : kMaxModes - 1;
@@ -921,16 +900,18 @@ __global__ void __launch_bounds__(kOneWarps * kWarp, 1) k_pass_one(const PassArg
             RowOne<T> own{};
             if (FIRST) own = load_row_one<T, true>(a.Zn + (int64_t)a.rank_n[item.row] * W);
             T B[1] = {T(0)}, c[1] = {T(0)};
-            const int end = (int)(item.begin + item.len);  // nnz < 2^31
-            for (int j = (int)item.begin + lane; j - lane < end; j += U * kWarp) {
+            const int end = (int)(item.begin + item.len);
+            int j0 = (int)item.begin;
+            while (j0 < end) {
                 int32_t i0[U], i1[U];
                 T rv[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const bool in = j + u * kWarp < end;
-                    i0[u] = in ? ix0[j + u * kWarp] : -1;
-                    i1[u] = in ? ix1[j + u * kWarp] : 0;
-                    rv[u] = in ? a.res[j + u * kWarp] : T(0);
+                    const int k = u * kWarp + lane;
+                    const bool in = has_entry(j0, k, end);
+                    i0[u] = in ? ix0[j0 + k] : -1;
+                    i1[u] = in ? ix1[j0 + k] : 0;
+                    rv[u] = in ? a.res[j0 + k] : T(0);
                 }
                 RowOne<T> r0[U], r1[U];
 #pragma unroll
@@ -951,11 +932,13 @@ __global__ void __launch_bounds__(kOneWarps * kWarp, 1) k_pass_one(const PassArg
                         else
                             po += own.old * (r0[u].old * (n_lo > 1 ? r1[u].old : r1[u].cur));
                         v = v - pp + po;
-                        a.res[j + u * kWarp] = v;
+                        a.res[j0 + (u * kWarp + lane)] = v;
                     }
                     c[0] += v * h;
                     B[0] += h * h;
                 }
+                if (last_step(j0, U * kWarp, end)) break;
+                j0 += U * kWarp;
             }
             Step st{};
             st.it = (int32_t)it;
@@ -1190,8 +1173,8 @@ struct ResConsumer {
         }
     }
     __device__ __forceinline__ void entry(const SM &sm, const Step &st, int rs, int is, int lane) {
+        if (!has_entry(st.j0, lane, st.jend)) return;
         const int j = st.j0 + lane;
-        if (j >= st.jend) return;
         T p = T(0);
         if (a.Cq > 0) {
             const T *slot = sm.rows(rs);

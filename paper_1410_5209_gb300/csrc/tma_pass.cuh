@@ -199,27 +199,12 @@ __global__ void __launch_bounds__(kTmaMaxWarps * kWarp, 1)
         return ib_items[it - ib_base];
     };
     auto step_at = [&](int64_t it) {
-        Step s;
-        s.it = (int32_t)it;
-        if (it >= it1) {
-            s.j0 = s.jend = 0;
-            s.flags = 0;
-            return s;
-        }
-        const tf_item &x = item_at(it);
-        s.j0 = (int32_t)x.begin;
-        s.jend = (int32_t)(x.begin + x.len);
-        s.flags = 1 | 2 | ((x.len <= kWarp) ? 4 : 0);
-        return s;
+        if (it >= it1) return no_step(it);
+        return first_step(item_at(it), it);
     };
     auto step_after = [&](const Step &s) {
         if (!(s.flags & 1)) return s;
-        if (s.j0 + kWarp < s.jend) {
-            Step n = s;
-            n.j0 += kWarp;
-            n.flags = 1 | ((n.j0 + kWarp >= n.jend) ? 4 : 0);
-            return n;
-        }
+        if (!(s.flags & 4)) return step_on(s);
         return step_at((int64_t)s.it + 1);
     };
 
@@ -343,8 +328,8 @@ __global__ void __launch_bounds__(kTmaMaxWarps * kWarp, 1)
                               : reinterpret_cast<const T *>(rslot(rs) + (t ? L.mode1_off : 0u)) +
                                     pos * ta.box[t];
             }
-            const int j = cur.j0 + lane;
             if (lane < nvalid) {
+                const int j = cur.j0 + lane;
                 T h[CM], po = T(0), pp = T(0);
                 // own = the own slice row: prev at CM, old at 2 CM
                 entry_products<T, CM, 2, FIRST, CM, 2 * CM>(rowp, own, 2, n_lo, C, Cq, h, po, pp);
