@@ -87,28 +87,30 @@ __device__ __forceinline__ T warp_sum(T v) {
     return v;
 }
 
-// How the Cholesky keeps its pivots and divides by them.  Double: inverted once per column,
-// since an FP64 division is a dozen instructions of the FP64 unit, which issues a warp's
-// instruction over 64 cycles.  Float: the square root and true divisions (the rounding of
-// every float row stays that of the plain formula).
+// v / pivot.  Float: the division.  Double: an FP64 division is a dozen instructions of the
+// FP64 unit, which issues a warp's instruction over 64 cycles, so the pivot is inverted once
+// per column and a quotient is the product with the rounded inverse, corrected by what it
+// leaves of v (three instructions; Markstein, "Computation of elementary functions on the IBM
+// RISC System/6000 processor", IBM J. Res. Dev. 34, 1990), which rounds as the division does.
+// The product alone took factors of a weighted-lambda fit from 1.6e-17 to 1.2e-15 off 64-bit
+// results.  Quotients that are zero, subnormal or not finite stay as the product gives them.
 template <class T>
-__device__ __forceinline__ T chol_pivot(T root) {
-    if constexpr (sizeof(T) == 8) return T(1) / root;
-    return root;
-}
-template <class T>
-__device__ __forceinline__ T chol_over(T v, T pivot) {
-    if constexpr (sizeof(T) == 8) return v * pivot;
+__device__ __forceinline__ T chol_over(T v, T pivot, T inverse) {
+    if constexpr (sizeof(T) == 8) {
+        const T q = v * inverse;
+        const unsigned e = (unsigned)__double2hiint(q) & 0x7FF00000u;
+        return e - 0x00100000u < 0x7FE00000u ? fma(fma(-q, pivot, v), inverse, q) : q;
+    }
     return v / pivot;
 }
 
 // Cholesky factor, in place, of B + lam I for the leading C x C block of a CM x CM packed
-// lower triangle; rows/columns >= C are replaced by the identity.  The diagonal holds
-// chol_pivot(L_jj).  min_ratio receives the smallest pivot ratio d_j / (B_jj + lam) over the
-// leading block (1 when perfectly conditioned, near 0 when a column is nearly a combination
-// of the earlier ones).  Returns false when a pivot is <= 0.
+// lower triangle; rows/columns >= C are replaced by the identity.  inv: inverses of the
+// factor's diagonal (double only).  min_ratio receives the smallest pivot ratio d_j / (B_jj +
+// lam) over the leading block (1 when perfectly conditioned, near 0 when a column is nearly a
+// combination of the earlier ones).  Returns false when a pivot is <= 0.
 template <class T, int CM>
-__device__ __forceinline__ bool chol_factor(T (&B)[CM * (CM + 1) / 2], int C, T lam,
+__device__ __forceinline__ bool chol_factor(T (&B)[CM * (CM + 1) / 2], T (&inv)[CM], int C, T lam,
                                             T &min_ratio) {
 #pragma unroll
     for (int i = 0; i < CM; ++i) {
@@ -135,8 +137,9 @@ __device__ __forceinline__ bool chol_factor(T (&B)[CM * (CM + 1) / 2], int C, T 
             if (k < j) d -= B[tri(j, k)] * B[tri(j, k)];
         ok = ok && (d > T(0));
         if (a_jj > T(0)) min_ratio = fmin(min_ratio, d / a_jj);
-        const T piv = chol_pivot<T>(sqrt(d > T(0) ? d : T(1)));
+        const T piv = sqrt(d > T(0) ? d : T(1));
         B[tri(j, j)] = piv;
+        inv[j] = sizeof(T) == 8 ? T(1) / piv : T(0);
 #pragma unroll
         for (int i = 0; i < CM; ++i) {
             if (i <= j) continue;
@@ -144,7 +147,7 @@ __device__ __forceinline__ bool chol_factor(T (&B)[CM * (CM + 1) / 2], int C, T 
 #pragma unroll
             for (int k = 0; k < CM; ++k)
                 if (k < j) s -= B[tri(i, k)] * B[tri(j, k)];
-            B[tri(i, j)] = chol_over<T>(s, piv);
+            B[tri(i, j)] = chol_over<T>(s, piv, inv[j]);
         }
     }
     return ok;
@@ -152,22 +155,22 @@ __device__ __forceinline__ bool chol_factor(T (&B)[CM * (CM + 1) / 2], int C, T 
 
 // x = (L L^T)^-1 r with the factor of chol_factor (r beyond C is ignored).
 template <class T, int CM>
-__device__ __forceinline__ void chol_apply(const T (&L)[CM * (CM + 1) / 2], const T (&r)[CM],
-                                           int C, T (&x)[CM]) {
+__device__ __forceinline__ void chol_apply(const T (&L)[CM * (CM + 1) / 2], const T (&inv)[CM],
+                                           const T (&r)[CM], int C, T (&x)[CM]) {
     T y[CM];
 #pragma unroll
     for (int i = 0; i < CM; ++i) {
         T s = (i < C) ? r[i] : T(0);
 #pragma unroll
         for (int k = 0; k < i; ++k) s -= L[tri(i, k)] * y[k];
-        y[i] = chol_over<T>(s, L[tri(i, i)]);
+        y[i] = chol_over<T>(s, L[tri(i, i)], inv[i]);
     }
 #pragma unroll
     for (int i = CM - 1; i >= 0; --i) {
         T s = y[i];
 #pragma unroll
         for (int k = i + 1; k < CM; ++k) s -= L[tri(k, i)] * x[k];
-        x[i] = chol_over<T>(s, L[tri(i, i)]);
+        x[i] = chol_over<T>(s, L[tri(i, i)], inv[i]);
     }
 }
 
@@ -177,9 +180,9 @@ __device__ __forceinline__ void chol_apply(const T (&L)[CM * (CM + 1) / 2], cons
 template <class T, int CM>
 __device__ __forceinline__ bool chol_solve(T (&B)[CM * (CM + 1) / 2], const T (&c)[CM], int C,
                                            T lam, T (&x)[CM]) {
-    T ratio;
-    const bool ok = chol_factor<T, CM>(B, C, lam, ratio);
-    chol_apply<T, CM>(B, c, C, x);
+    T ratio, inv[CM];
+    const bool ok = chol_factor<T, CM>(B, inv, C, lam, ratio);
+    chol_apply<T, CM>(B, inv, c, C, x);
     return ok;
 }
 
@@ -196,8 +199,8 @@ __device__ __forceinline__ bool row_solve(const PassArgs<T> &a, const T (&B)[CM 
     T L[NT];
 #pragma unroll
     for (int q = 0; q < NT; ++q) L[q] = B[q];
-    T ratio;
-    bool ok = chol_factor<T, CM>(L, C, lam, ratio);
+    T ratio, inv[CM];
+    bool ok = chol_factor<T, CM>(L, inv, C, lam, ratio);
     if constexpr (sizeof(T) == 4) {
         if (a.cond_limit > 0.f && (!ok || ratio * a.cond_limit < 1.f)) {
             double Bd[NT], cd[CM], xd[CM];
@@ -212,7 +215,7 @@ __device__ __forceinline__ bool row_solve(const PassArgs<T> &a, const T (&B)[CM 
             return true;
         }
         if (!ok) return false;
-        chol_apply<T, CM>(L, c, C, x);
+        chol_apply<T, CM>(L, inv, c, C, x);
         if (a.refine) {
             T r[CM], dx[CM];
 #pragma unroll
@@ -225,13 +228,13 @@ __device__ __forceinline__ bool row_solve(const PassArgs<T> &a, const T (&B)[CM 
                 }
                 r[i] = (T)s;
             }
-            chol_apply<T, CM>(L, r, C, dx);
+            chol_apply<T, CM>(L, inv, r, C, dx);
 #pragma unroll
             for (int i = 0; i < CM; ++i) x[i] += dx[i];
         }
         return true;
     } else {
-        if (ok) chol_apply<T, CM>(L, c, C, x);
+        if (ok) chol_apply<T, CM>(L, inv, c, C, x);
         return ok;
     }
 }
