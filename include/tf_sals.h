@@ -261,7 +261,9 @@ tf_status tf_foldin(tf_ctx *ctx, int mode, const int32_t *other, const void *val
  * coordinates, e.g. held-out entries for a test RMSE.
  *   coords [m][N] int32, 0-based; out [m] context dtype.  Both host buffers, or both
  *   device buffers on the context's device with flags = TF_INPUT_DEVICE.
- * Products and the sum over k in double on the device.  Synchronises.  TF_ERANGE if a
+ * Products and the sum over k in double on the device, in float contexts in pairs of floats
+ * (about 48 bits) where the terms' range and cancellation leave a float result the same
+ * accuracy.  Synchronises.  TF_ERANGE if a
  * coordinate is out of range (out is then unspecified). */
 tf_status tf_predict(tf_ctx *ctx, const int32_t *coords, int64_t m, void *out, uint32_t flags);
 

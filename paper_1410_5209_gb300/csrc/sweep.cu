@@ -206,11 +206,18 @@ __global__ void k_init_normal(T *A, int64_t count, uint64_t key, double std) {
 //   FP64 unit (three conversions, two products and a sum per column at 1/64 of the FP32
 //   rate) and left 22% of its lanes idle at K = 100.  8 lanes per coordinate with 16-byte
 //   loads keep 4 N loads per lane in flight at K = 100.  3,000,017 coordinates, N = 3,
-//   K = 100 on GB300: 6.11 ms before, 0.63 ms now
-//   (5.7 TB/s of gathered rows).
-// A pair loses bits where a product or its error leaves the float range, so a coordinate
-// whose values reach a.big (2^(56 / (N - 1)): no product overflows) or whose sum is below
-// 2^-40 or not finite is formed again in FP64 (redo).
+//   K = 100 on GB300: 6.11 ms before, 0.62 ms now
+//   (5.8 TB/s of gathered rows).
+// A pair loses bits where a product or its error leaves the float range, and a sum of pairs
+// keeps 2^-40 of the terms' magnitudes at worst (Ogita, Rump and Oishi: the square of 2^-24
+// times the additions in a chain; 2^-46 is usual) where FP64 keeps 2^-53.  So a coordinate is
+// formed again in FP64 whose values reach a.big (2^(56 / (N - 1)): no product overflows), whose
+// sum is below 2^-40 or not finite, or whose terms cancel to less than 2^-13 of their
+// magnitudes (below that line the worst error is an eighth of the result's rounding; 1 of 1,000
+// coordinates with terms of random sign, K = 100).  A sum all of whose terms have a zero factor
+// (rows without entries solve to zero) is exact as it is, which a second look at the factors
+// shows where the magnitudes' sum is zero: with 30% of the rows of one mode zero 0.70 ms, and
+// 3.39 when those took the FP64 form too.
 template <class T>
 struct PredictVec;
 template <>
@@ -276,7 +283,7 @@ __global__ void __launch_bounds__(256) k_predict(const PredictArgs<T> a) {
     };
     if constexpr (sizeof(T) == 4) {
         FloatPair sum[V];
-        float big = 0.f;
+        float big = 0.f, mag = 0.f;  // largest factor, sum of the terms' magnitudes
 #pragma unroll
         for (int u = 0; u < V; ++u) sum[u].h = sum[u].l = 0.f;
 #pragma unroll 4
@@ -300,12 +307,33 @@ __global__ void __launch_bounds__(256) k_predict(const PredictArgs<T> a) {
             }
 #pragma unroll
             for (int u = 0; u < V; ++u) pair_add(sum[u], p[u].h, p[u].l);
+            if constexpr (V == 4)
+                mag += (fabsf(p[0].h) + fabsf(p[1].h)) + (fabsf(p[2].h) + fabsf(p[3].h));
+            else
+                mag += fabsf(p[0].h);
         }
 #pragma unroll
         for (int u = 1; u < V; ++u) pair_add(sum[0], sum[u].h, sum[u].l);
         const FloatPair s = pair_group_sum(sum[0], LP, mask);
+#pragma unroll
+        for (int o = LP / 2; o > 0; o >>= 1) mag += __shfl_xor_sync(mask, mag, o);
         float r = __fadd_rn(s.h, s.l);
-        const bool fine = big < a.big && fabsf(r) >= 0x1p-40f && fabsf(r) < 0x1p126f;
+        bool fine = big < a.big && fabsf(r) >= 0x1p-40f && fabsf(r) < 0x1p126f &&
+                    mag <= 0x1p13f * fabsf(r);
+        if (mag == 0.f) {  // zero factors, or products that vanished?
+            fine = true;
+            for (int k = sub * V; k < a.K; k += LP * V) {
+                float v[V], least[V];
+                load(0, k, least);
+                for (int n = 1; n < N; ++n) {
+                    load(n, k, v);
+#pragma unroll
+                    for (int u = 0; u < V; ++u) least[u] = fminf(fabsf(least[u]), fabsf(v[u]));
+                }
+#pragma unroll
+                for (int u = 0; u < V; ++u) fine = fine && least[u] == 0.f;
+            }
+        }
         if (__any_sync(mask, !fine)) r = (float)predict_f64<T, LP>(a, c, sub, mask);
         if (sub == 0) a.out[e] = r;
     } else {
