@@ -146,7 +146,11 @@ __global__ void __launch_bounds__(kFoldThreads) k_foldin(const FoldArgs<T> a) {
 //     the factor.
 //   k_fold_resid (float): sum_e h_e (x_e - h_e . x0) in pairs of floats (float_pair.cuh,
 //     ~48 bits; in FP64 it took 8 times as long), 8 lanes per entry, then the correction
-//     solved with the stored factor.
+//     solved with the stored factor.  One step of refinement leaves 2^-48 times the square of
+//     the condition, so pairs do for it what FP64 does (condition 2e0 to 6e4: errors of the
+//     rows 2e-8 to 9e-8, with the former FP64 residual 2e-8 to 3e-7) as long as no bits fall
+//     out of the float range: a block that meets a nonzero product or value below 2^-40, or
+//     whose sums are not finite, forms its sums in FP64.
 // Bad indices and non-positive pivots are flagged per request in req_status (1 and 2).
 constexpr int kFoldTile = 32;
 constexpr int kFoldBlock = 256;  // two blocks an SM at 128 registers
@@ -587,6 +591,54 @@ __host__ __device__ constexpr size_t fold_resid_smem(int K) {
     return red > solve ? red : solve;
 }
 
+// With |h| and |x| from here on (or zero), an error term lost below 2^-149 is at most 2^-69 of
+// h x.
+constexpr float kFoldLeast = 0x1p-40f;
+
+// The warps' sums of h_e (x_e - h_e . x0) in FP64, lanes and columns as in k_fold_resid; x: the
+// lane's columns of x0.
+template <int R>
+__device__ __noinline__ void fold_resid_f64(const FoldArgs<float> &a,
+                                            const float (&x)[FoldCols<float, R>::N], int64_t b0,
+                                            int64_t b1, double *sums) {
+    using FC = FoldCols<float, R>;
+    const int K = a.K, grp = threadIdx.x >> 3, g = threadIdx.x & 7;
+    const bool vec = fold_vec<float, R>(K);
+    double acc[FC::N];
+#pragma unroll
+    for (int j = 0; j < FC::N; ++j) acc[j] = 0.0;
+    for (int64_t e0 = b0; e0 < b1; e0 += 32) {
+        const bool valid = e0 + grp < b1;
+        const int64_t es = valid ? e0 + grp : b0;
+        double h[FC::N], dot = 0.0;
+#pragma unroll
+        for (int j = 0; j < FC::N; ++j) h[j] = 1.0;
+        for (int t = 0; t < a.N - 1; ++t) {
+            const int l = t < a.mode ? t : t + 1;
+            float v[FC::N];
+            FC::row(a.A[l] + (int64_t)a.other[es * (a.N - 1) + t] * K, K, g, vec, v);
+#pragma unroll
+            for (int j = 0; j < FC::N; ++j) h[j] *= (double)v[j];
+        }
+#pragma unroll
+        for (int j = 0; j < FC::N; ++j)
+            if (FC::col(j, g, vec) < K) dot += h[j] * (double)x[j];
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) dot += __shfl_xor_sync(0xFFFFFFFFu, dot, o);
+        const double rho = (double)a.x[es] - dot;
+        if (valid)
+#pragma unroll
+            for (int j = 0; j < FC::N; ++j) acc[j] += h[j] * rho;
+    }
+#pragma unroll
+    for (int j = 0; j < FC::N; ++j) {
+        const int c = FC::col(j, g, vec);
+#pragma unroll
+        for (int o = 8; o < 32; o <<= 1) acc[j] += __shfl_xor_sync(0xFFFFFFFFu, acc[j], o);
+        if ((grp & 3) == 0 && c < K) sums[(grp >> 2) * K + c] = acc[j];
+    }
+}
+
 template <int R, int NO>
 __global__ void __launch_bounds__(kFoldBlock) k_fold_resid(const FoldArgs<float> a) {
     using FC = FoldCols<float, R>;
@@ -608,6 +660,7 @@ __global__ void __launch_bounds__(kFoldBlock) k_fold_resid(const FoldArgs<float>
         x[j] = c < K ? x0[c] : 0.f;
     }
     FloatPair acc[FC::N];
+    bool lost = false;  // a product or value outside the pairs' range
 #pragma unroll
     for (int j = 0; j < FC::N; ++j) acc[j].h = acc[j].l = 0.f;
     for (int64_t e0 = b0; e0 < b1; e0 += 32) {
@@ -626,12 +679,18 @@ __global__ void __launch_bounds__(kFoldBlock) k_fold_resid(const FoldArgs<float>
             FC::row(a.A[l] + (int64_t)idx * K, K, g, vec, v);
 #pragma unroll
             for (int j = 0; j < FC::N; ++j) {
-                if (t == 0)
+                if (t == 0) {
                     h[j].h = v[j];
-                else
+                    lost = lost || (no == 1 && fabsf(v[j]) < kFoldLeast && v[j] != 0.f);
+                } else {
+                    const float before = h[j].h;
                     h[j] = pair_mul(h[j], v[j]);
+                    lost = lost || (fabsf(h[j].h) < kFoldLeast && before != 0.f && v[j] != 0.f);
+                }
             }
         }
+        const float xe = a.x[es];
+        lost = lost || (fabsf(xe) < kFoldLeast && xe != 0.f);
         FloatPair dot = {0.f, 0.f};
 #pragma unroll
         for (int j = 0; j < FC::N; ++j)
@@ -641,7 +700,7 @@ __global__ void __launch_bounds__(kFoldBlock) k_fold_resid(const FoldArgs<float>
             }
         dot = pair_group_sum(dot, 8, 0xFFFFFFFFu);
         FloatPair rho;
-        rho.h = two_sum(a.x[es], -dot.h, rho.l);
+        rho.h = two_sum(xe, -dot.h, rho.l);
         rho.l = __fsub_rn(rho.l, dot.l);
         if (valid)
 #pragma unroll
@@ -652,15 +711,22 @@ __global__ void __launch_bounds__(kFoldBlock) k_fold_resid(const FoldArgs<float>
             }
     }
 #pragma unroll
-    for (int j = 0; j < FC::N; ++j) {
-        // the warp's four groups, still as pairs; then one row of doubles per warp
-        const int c = FC::col(j, g, vec);
+    for (int j = 0; j < FC::N; ++j)
+        lost = lost || !(fabsf(acc[j].h) + fabsf(acc[j].l) < INFINITY);
+    if (!__syncthreads_or(lost)) {
 #pragma unroll
-        for (int o = 8; o < 32; o <<= 1)
-            pair_add(acc[j], __shfl_xor_sync(0xFFFFFFFFu, acc[j].h, o),
-                     __shfl_xor_sync(0xFFFFFFFFu, acc[j].l, o));
-        if ((grp & 3) == 0 && c < K)
-            sums[(grp >> 2) * K + c] = (double)acc[j].h + (double)acc[j].l;
+        for (int j = 0; j < FC::N; ++j) {
+            // the warp's four groups, still as pairs; then one row of doubles per warp
+            const int c = FC::col(j, g, vec);
+#pragma unroll
+            for (int o = 8; o < 32; o <<= 1)
+                pair_add(acc[j], __shfl_xor_sync(0xFFFFFFFFu, acc[j].h, o),
+                         __shfl_xor_sync(0xFFFFFFFFu, acc[j].l, o));
+            if ((grp & 3) == 0 && c < K)
+                sums[(grp >> 2) * K + c] = (double)acc[j].h + (double)acc[j].l;
+        }
+    } else {
+        fold_resid_f64<R>(a, x, b0, b1, sums);
     }
     __syncthreads();
     for (int k = tid; k < K; k += kFoldBlock) {
