@@ -1912,12 +1912,30 @@ struct Impl : CtxBase {
         f_other.ensure((size_t)std::max<int64_t>(m, 1) * std::max(N - 1, 1), st);
         f_x.ensure((size_t)std::max<int64_t>(m, 1), st);
         f_out.ensure((size_t)n_req * K, st);
-        f_part.ensure(foldin_part_elems(K, blocks), st);
         const bool refine = sizeof(T) == 4;
+        // launches: groups of consecutive requests with bounded scratch, which each group
+        // uses in turn (a request's row does not depend on its group)
+        auto scratch = [&](int r0, int r1, size_t &part, size_t &rpart, size_t &fac) {
+            part = foldin_part_elems(K, req_blk[r1] - req_blk[r0]);
+            rpart = fac = 0;
+            if (refine) rpart = foldin_refine_elems(K, req_blk[r1] - req_blk[r0], r1 - r0, &fac);
+            return (part + fac) * sizeof(T) + rpart * sizeof(double);
+        };
+        std::vector<int> group{0};
+        size_t part, rpart, fac, part_most = 0, rpart_most = 0, fac_most = 0;
+        for (int r = 0; r < n_req; ++r) {
+            if (r > group.back() && scratch(group.back(), r + 1, part, rpart, fac) > kFoldScratch)
+                group.push_back(r);
+            scratch(group.back(), r + 1, part, rpart, fac);
+            part_most = std::max(part_most, part);
+            rpart_most = std::max(rpart_most, rpart);
+            fac_most = std::max(fac_most, fac);
+        }
+        group.push_back(n_req);
+        f_part.ensure(part_most, st);
         if (refine) {
-            size_t fac_elems = 0;
-            f_rpart.ensure(foldin_refine_elems(K, blocks, n_req, &fac_elems), st);
-            f_fac.ensure(fac_elems, st);
+            f_rpart.ensure(rpart_most, st);
+            f_fac.ensure(fac_most, st);
         }
         // one int64 staging buffer: block entry ranges [2B], then as int32 the blocks'
         // requests [B], the requests' first blocks [n_req + 1], their status [n_req] and two
@@ -1963,7 +1981,11 @@ struct Impl : CtxBase {
         a.refine = refine ? 1 : 0;
         a.fac = refine ? f_fac.p : nullptr;
         a.rpart = refine ? f_rpart.p : nullptr;
-        launch_foldin_tiled<T>(a, blocks, st);
+        for (size_t q = 0; q + 1 < group.size(); ++q) {
+            a.req0 = group[q];
+            a.blk0 = req_blk[group[q]];
+            launch_foldin_tiled<T>(a, req_blk[group[q + 1]] - a.blk0, st);
+        }
         std::vector<T> rows((size_t)n_req * K);
         TFS_CUDA(cudaMemcpyAsync(status, a.req_status, (size_t)n_req * sizeof(int32_t),
                                  cudaMemcpyDeviceToHost, st));

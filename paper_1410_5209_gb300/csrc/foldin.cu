@@ -467,8 +467,8 @@ __global__ void __launch_bounds__(kFoldBlock, sizeof(T) == 4 ? 2 : 1)
     for (int i = 0; i < R; ++i)
 #pragma unroll
         for (int j = 0; j < R; ++j) acc[i][j] = T(0);
-    const int req = a.blk_req[blockIdx.x];
-    const int64_t b0 = a.blk_range[2 * blockIdx.x], b1 = a.blk_range[2 * blockIdx.x + 1];
+    const int blk = a.blk0 + blockIdx.x, req = a.blk_req[blk];
+    const int64_t b0 = a.blk_range[2 * blk], b1 = a.blk_range[2 * blk + 1];
     for (int64_t e0 = b0; e0 < b1; e0 += kFoldTile) {
         const int ne = (int)(b1 - e0 < kFoldTile ? b1 - e0 : kFoldTile);
         const int e = tid >> 3, g = tid & 7;
@@ -546,7 +546,7 @@ __global__ void __launch_bounds__(kFoldBlock, sizeof(T) == 4 ? 2 : 1)
     for (int q0 = tid; q0 < PB; q0 += 4 * kFoldBlock) {
         T s[4] = {T(0), T(0), T(0), T(0)};
         for (int b = bb; b < be; ++b) {
-            const T *p = a.part + (int64_t)b * PB;
+            const T *p = a.part + (int64_t)(b - a.blk0) * PB;
 #pragma unroll
             for (int u = 0; u < 4; ++u)
                 if (q0 + u * kFoldBlock < PB) s[u] += __ldcg(p + q0 + u * kFoldBlock);
@@ -571,7 +571,7 @@ __global__ void __launch_bounds__(kFoldBlock, sizeof(T) == 4 ? 2 : 1)
     for (int k = tid; k < K; k += kFoldBlock) a.out[(int64_t)req * K + k] = y[k];
     if (a.refine) {
         const int LF = fold_fac_ld(K), V = 16 / (int)sizeof(T), nv = LF / V;
-        T *f = a.fac + (int64_t)req * K * LF;
+        T *f = a.fac + (int64_t)(req - a.req0) * K * LF;
         using Q = typename FoldVec<T>::type;
         for (int q = tid; q < K * nv; q += kFoldBlock) {
             const int r = q / nv, v = q - r * nv;
@@ -645,12 +645,12 @@ __global__ void __launch_bounds__(kFoldBlock) k_fold_resid(const FoldArgs<float>
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int flag;
     const int tid = threadIdx.x, K = a.K;
-    const int req = a.blk_req[blockIdx.x];
+    const int blk = a.blk0 + blockIdx.x, req = a.blk_req[blk];
     if (a.req_status[req] != 0) return;  // bad index or pivot: every block of it leaves
     const bool vec = fold_vec<float, R>(K);
     const float *x0 = a.out + (int64_t)req * K;
     double *sums = reinterpret_cast<double *>(smem_raw);
-    const int64_t b0 = a.blk_range[2 * blockIdx.x], b1 = a.blk_range[2 * blockIdx.x + 1];
+    const int64_t b0 = a.blk_range[2 * blk], b1 = a.blk_range[2 * blk + 1];
     const int grp = tid >> 3, g = tid & 7;
     const int no = NO > 0 ? NO : a.N - 1;
     float x[FC::N];
@@ -740,7 +740,7 @@ __global__ void __launch_bounds__(kFoldBlock) k_fold_resid(const FoldArgs<float>
     const int LD = fold_ld<float>(K), LF = fold_fac_ld(K), nv = LF / 4;
     float *A = reinterpret_cast<float *>(smem_raw), *d = A + K * LD, *invd = d + 128,
           *red = invd + 128;
-    const float *f = a.fac + (int64_t)req * K * LF;
+    const float *f = a.fac + (int64_t)(req - a.req0) * K * LF;
     for (int q = tid; q < K * nv; q += kFoldBlock) {
         const int r = q / nv, v = q - r * nv;
         if (4 * v <= r)
@@ -749,7 +749,7 @@ __global__ void __launch_bounds__(kFoldBlock) k_fold_resid(const FoldArgs<float>
     }
     for (int k = tid; k < K; k += kFoldBlock) {
         double s = 0.0;
-        for (int b = bb; b < be; ++b) s += __ldcg(a.rpart + (int64_t)b * K + k);
+        for (int b = bb; b < be; ++b) s += __ldcg(a.rpart + (int64_t)(b - a.blk0) * K + k);
         d[k] = (float)(s - (double)a.lambda * (double)x0[k]);
     }
     __syncthreads();
@@ -781,7 +781,8 @@ void launch_foldin_edge(const FoldArgs<T> &a, int blocks, cudaStream_t st) {
 bool foldin_tiled_ok(int K) { return K + 1 <= 128; }
 
 // Blocks of a request of m entries: 64 entries each up to 1,024 (a lone request then spreads
-// over up to 16 SMs), 256 beyond (fewer partial systems to write and sum).  A request
+// over up to 16 SMs), 256 beyond (fewer partial systems to write and sum): up to 370 KB of
+// partial systems a request of 1,024 entries at K = 100.  A request
 // without entries has one empty block, which solves lambda I x = 0.
 int foldin_plan_blocks(const int64_t *offsets, int n_req, std::vector<int64_t> &blk_range,
                        std::vector<int32_t> &blk_req, std::vector<int32_t> &req_blk) {

@@ -147,18 +147,20 @@ struct FoldArgs {
     T lambda;
     T *out;
     DeviceStatus *stat;
-    T *part;      // [blocks] partial Gram / rhs tiles of the tiled fold-in
+    T *part;      // [blocks of the launch] partial Gram / rhs tiles of the tiled fold-in
     // tiled fold-in of a batch: per block its entry range and request, per request its
     // first block (n_req + 1), a status word (1 bad index, 2 bad pivot) and two counts of
-    // finished blocks (req_count [2][n_req], zero on entry); out is then [n_req][K]
-    int n_req;
+    // finished blocks (req_count [2][n_req], zero on entry); out is then [n_req][K].  A
+    // launch takes the requests from req0 on, whose blocks start at blk0.
+    int n_req, req0, blk0;
     const int64_t *blk_range;
     const int32_t *blk_req;
     const int32_t *req_blk;
     int32_t *req_status;
     int32_t *req_count;
     // float contexts: one step of iterative refinement of every request's solve.  The
-    // solve keeps its Cholesky factor in fac [n_req] (rows of K rounded up to 4); a second
+    // solve keeps its Cholesky factor in fac (per request of the launch, rows of K rounded up
+    // to 4); a second
     // pass over the request's entries forms the residual of the normal equations,
     // c - (B + lambda I) x0 = sum_e h_e (x_e - h_e . x0) - lambda x0, to twice the working
     // precision (per-block partials in rpart [blocks][K], FP64); the correction solved with
@@ -306,7 +308,9 @@ struct PredictArgs {
 template <class T>
 void launch_predict(const PredictArgs<T> &a, cudaStream_t st);
 // Tiled fold-in (K < 128): block table of a batch of requests (offsets[n_req + 1] into
-// the concatenated entries), partial buffer length, launch.
+// the concatenated entries), partial buffer length, launch.  Scratch is bounded: a batch goes
+// in groups of requests that stay within kFoldScratch (or of one request that does not).
+constexpr size_t kFoldScratch = size_t(64) << 20;
 bool foldin_tiled_ok(int K);
 int foldin_plan_blocks(const int64_t *offsets, int n_req, std::vector<int64_t> &blk_range,
                        std::vector<int32_t> &blk_req, std::vector<int32_t> &req_blk);
