@@ -711,11 +711,6 @@ LeanPlan lean_pass_plan(int CM, bool first, int n, const int64_t *dims_o,
         R[best] += best_rows;
         used += (size_t)best_rows * csw[best] * 4;
     }
-    {
-        const int var = 1 - lean_run_mode(n);
-        const std::vector<int64_t> &dc = *deg_cum[var];
-        pl.coverage = nnz > 0 ? (double)dc[R[var]] / (double)nnz : 1.0;
-    }
     pl.grid = std::max(1, std::min(num_sms, (P + pl.warps - 1) / pl.warps));
     // every block copies the cached rows: a row with fewer entries than there are blocks is
     // gathered less often than it would be copied (rows are in decreasing order of entries;
@@ -736,6 +731,15 @@ LeanPlan lean_pass_plan(int CM, bool first, int n, const int64_t *dims_o,
             }
             R[t] = lo;
         }
+    // what the cache serves, which decides between this pass and the staged one: rows that are
+    // not worth their copies leave nothing here (three passes of 700^3, 1e5 entries, C = 4 / 10:
+    // 16.3 / 22.8 us each with empty caches, 13.3 / 14.9 in the staged pass; 12,000^3, 1.6e6,
+    // C = 4: 54 and 45; the other way only below 5e4 entries, 3,000^3, 4e4: 11.5 and 14.3)
+    {
+        const int var = 1 - lean_run_mode(n);
+        const std::vector<int64_t> &dc = *deg_cum[var];
+        pl.coverage = nnz > 0 ? (double)dc[R[var]] / (double)nnz : 1.0;
+    }
     lp.R[0] = R[0];
     lp.R[1] = R[1];
     lp.cache_off[0] = 0;
