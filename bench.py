@@ -909,7 +909,9 @@ def main():
     roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                 "frac": achieved / hbm, "traffic": traffic,
                 "kernel": " + ".join(n for b, n in ((1, "k_pass_wide" if C > 16 else "k_mode_pass"),
-                                                   (2, "k_mode_pass_tma"), (4, "k_pass_wide_tc"),
+                                                   (2, "k_mode_pass_tma"),
+                                                   (4, "k_pass_mma" if cnt["pass_path"] & 16
+                                                    else "k_pass_wide_tc"),
                                                    (8, "k_lean_pass"))
                                      if cnt["pass_path"] & b) or "?",
                 "peak_source": peak_kind,

@@ -294,8 +294,8 @@ tf_status tf_get_residual(tf_ctx *ctx, void *host_r);
  * counters[3] = work items of all modes, counters[4] = rows split across bins,
  * counters[5] = bins P of the schedule, counters[6] = kernels launched by the last
  * tf_loss, counters[7] = mode-pass data paths the last sweep used (bit 0: SIMT pass,
- * bit 1: TMA gather pass, bit 2: tensor-core Gram pass of wide subsets, with bit 0 where a
- * SIMT kernel stands behind it; 0 = no sweep). */
+ * bit 1: TMA gather pass, bit 2: tensor-core Gram pass of wide subsets, bit 3: lean pass,
+ * bit 4, with bit 2: the wide pass with register operands; 0 = no sweep). */
 tf_status tf_get_counters(tf_ctx *ctx, int64_t counters[8]);
 
 /* Re-plans the row schedule of every mode (policy, P bins; P = 0 picks the default

@@ -242,7 +242,10 @@ struct Impl : CtxBase {
     ModeLayout mode[kMaxModes];
     Buf<T> partials;
     Buf<int32_t> d_order, d_Q;
-    Buf<uint32_t> wide_mx;  // largest current column values of wide sweeps (wide_max)
+    // gated wide sweeps: kRanWords counts of launches that worked (register pass, SIMT, tcgen05
+    // pass), then the largest current column values (wide_max)
+    Buf<uint32_t> wide_mx;
+    static constexpr int kRanWords = 4;
     Buf<DeviceStatus> stat;
     Buf<unsigned long long> ticket;  // bin counter of the mode passes
     unsigned long long ticket_base = 0;
@@ -298,7 +301,10 @@ struct Impl : CtxBase {
     bool dirty = false;            // residual copies must be rebuilt from the factors
     bool a0_zero = true;           // A^(1) known to be zero (R = X)
     int64_t sweeps = 0, last_launches = 0, loss_launches = 0;
-    int64_t last_path = 0;  // mode-pass paths of the last sweep: bit 0 cp.async, bit 1 TMA
+    // mode-pass paths of the last sweep (tf_get_counters); kPathGated: on the device, as the
+    // counts of wide_mx
+    int64_t last_path = 0;
+    static constexpr int64_t kPathGated = int64_t(1) << 32;
     int64_t launches = 0;
     int64_t layout_gen = 0;  // bumped whenever the row schedule is rebuilt
 
@@ -1139,10 +1145,13 @@ struct Impl : CtxBase {
         return d;
     }
 
-    // Largest |current column value| of mode l in split s: 0 after the pack, t + 1 after inner
+    // Largest |current column values| of mode l in split s: 0 after the pack, t + 1 after inner
     // iteration t (PassArgs::mx).
     uint32_t *wide_max(int s, int when, int l, int T_in) {
-        return wide_mx.p + ((size_t)s * (T_in + 1) + when) * N + l;
+        return wide_mx.p + kRanWords + (((size_t)s * (T_in + 1) + when) * N + l) * kGateCols;
+    }
+    size_t wide_max_words(int nsplit, int T_in) const {
+        return kRanWords + (size_t)nsplit * (T_in + 1) * N * kGateCols;
     }
 
     // ------------------------------------------------------------ the sweep
@@ -1234,14 +1243,14 @@ struct Impl : CtxBase {
         const bool wide_mma = sizeof(T) == 4 && wide && path != 1 && path != 2 && precision != 1 &&
                               pass_mma_supported(N, C, CM) &&
                               solve_mid_supported(C, solve_refine || solve_cond > 0.f);
-        if (wide_mma) wide_mx.ensure((size_t)nsplit * (T_in + 1) * N, st);
+        if (wide_mma) wide_mx.ensure(wide_max_words(nsplit, T_in), st);
         // every launch of the splits (pack, mode passes, solves) and the copy of the last
         // split's columns into Q; returns |Q|
         auto run_splits = [&]() {
             int cq = Cq;
             if (wide_mma)
-                TFS_CUDA(cudaMemsetAsync(wide_mx.p, 0, (size_t)nsplit * (T_in + 1) * N * sizeof(uint32_t),
-                                         st));
+                TFS_CUDA(cudaMemsetAsync(wide_mx.p, 0,
+                                         wide_max_words(nsplit, T_in) * sizeof(uint32_t), st));
             const int32_t *Qp = d_Q.p;
             for (int s = 0; s < nsplit; ++s) {
                 const int Cs = (s == nsplit - 1) ? K - s * C : C;
@@ -1325,6 +1334,7 @@ struct Impl : CtxBase {
                                     }
                                     a.mx_out = wide_max(s, t + 1, n, T_in);
                                     a.gate = 1;
+                                    a.ran = wide_mx.p;
                                     a.gate_tickets = (unsigned long long)L.P +
                                                      (unsigned long long)plan.grid * plan.warps;
                                     timed(TF_KIND_MODE_PASS,
@@ -1332,7 +1342,8 @@ struct Impl : CtxBase {
                                     ticket_base += a.gate_tickets;
                                     a.ticket_base = ticket_base;
                                     a.gate = 2;
-                                    last_path |= 4;
+                                    a.ran = wide_mx.p + (tc ? 2 : 1);
+                                    last_path = kPathGated;
                                     ++launches;
                                 }
                             }
@@ -1342,7 +1353,7 @@ struct Impl : CtxBase {
                             ticket_base += a.gate_tickets;
                             timed(TF_KIND_MODE_PASS,
                                   [&] { launch_pass_wide<T>(a, CM, W, wgrid, tc, precision != 1, st); });
-                            last_path |= tc ? 4 : 1;
+                            if (!wide_mma) last_path |= tc ? 4 : 1;
                             ++launches;
                             if constexpr (sizeof(T) == 4) {
                                 if (solve_mid_supported(Cs, solve_refine || solve_cond > 0.f)) {
@@ -2087,7 +2098,16 @@ struct Impl : CtxBase {
         c[4] = split;
         c[5] = P;
         c[6] = loss_launches;
-        c[7] = last_path;
+        c[7] = path_bits();
+    }
+
+    // The paths of the last sweep, read back where the device chose them.
+    int64_t path_bits() {
+        if (last_path != kPathGated) return last_path;
+        uint32_t ran[kRanWords];
+        TFS_CUDA(cudaMemcpyAsync(ran, wide_mx.p, sizeof(ran), cudaMemcpyDeviceToHost, st));
+        TFS_CUDA(cudaStreamSynchronize(st));
+        return (ran[0] ? 16 | 4 : 0) | (ran[1] ? 1 : 0) | (ran[2] ? 4 : 0);
     }
 
     // ------------------------------------------------------------ autotuning
@@ -2122,7 +2142,7 @@ struct Impl : CtxBase {
         const int Cq0 = Cq, CMl0 = CM_last;
         const bool dirty0 = dirty, a00 = a0_zero;
         const int64_t sweeps0 = sweeps, launches0 = launches, last0 = last_launches;
-        const int64_t path0 = last_path;
+        const int64_t path0 = path_bits();
         const int P0 = P;
         auto restore = [&] {
             for (int n = 0; n < N; ++n) {

@@ -253,8 +253,8 @@ __global__ void __launch_bounds__(kMidThreads) k_solve_mid(const PassArgs<float>
         }
     }
     if (a.mx_out) {
-        record_max(a.mx_out, in0 ? x0 : 0.f);
-        if (R == 2) record_max(a.mx_out, in1 ? x1 : 0.f);
+        if (in0) record_max(a.mx_out + lane, x0);
+        if (in1) record_max(a.mx_out + lane + 32, x1);
     }
 }
 

@@ -24,10 +24,11 @@
 // 2.0e-6, and 1.5e-6 with FP32 throughout.  With two chunks the FMAs' registers cost 0.2 ms of
 // 1.6, and the errors are a third of FP32's without them (dispatch in api.cu).
 //   Range.  Below 2^-100 the split of h would lose its last parts, and collapsed columns
-// (weighted lambda) do get there.  The pack and the solves record the largest value of every
-// mode's current columns (PassArgs::mx); a pass whose factors' product lies outside 2^-80 ..
-// 2^60 and is not zero is left to the block-wide kernel, launched behind this one with the
-// opposite gate (one of the two returns at once).
+// (weighted lambda) do get there.  The pack and the solves record the largest value of each of
+// every mode's current columns (PassArgs::mx); a pass in which some column's product lies
+// outside 2^-80 .. 2^60 and is not zero is left to the block-wide kernel, launched behind this
+// one with the opposite gate (one of the two returns at once).  No cost beside one maximum
+// over all columns (C = 20 and 50: solves and passes as they were, the pack 0.13 -> 0.08 ms).
 #include <algorithm>
 
 #include "entry_steps.h"

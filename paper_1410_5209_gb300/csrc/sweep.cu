@@ -53,28 +53,37 @@ constexpr int kPackThreads = 256;
 
 template <class T>
 __global__ void __launch_bounds__(kPackThreads) k_pack(const PackArgs<T> a) {
+    __shared__ uint32_t mx[kMaxModes * kGateCols];
     const int CM = a.off_prev, rows = kPackThreads / CM;
     const int w = (int)threadIdx.x / CM, c = (int)threadIdx.x - w * CM;
-    const int64_t r = (int64_t)blockIdx.x * rows + w;
-    const bool live = w < rows && r < a.row_base[a.N];
-    if (!a.mx && !live) return;
-    int l = 0;
-    while (live && r >= a.row_base[l + 1]) ++l;
-    if (a.mx) {  // wide float passes: largest value per mode (mostly one mode per warp)
-        const float v =
-            live && c < a.C ? (float)a.A[l][(int64_t)a.id_of[l][r - a.row_base[l]] * a.K + a.S[c]] : 0.f;
-        for (int m = 0; m < a.N; ++m)
-            if (__any_sync(0xFFFFFFFFu, live && l == m)) record_max(a.mx + m, l == m ? v : 0.f);
+    if (a.mx) {
+        for (int q = threadIdx.x; q < a.N * kGateCols; q += kPackThreads) mx[q] = 0u;
+        __syncthreads();
     }
-    if (!live) return;
-    const int64_t i = r - a.row_base[l];  // slice row (rank)
-    const T *Ar = a.A[l] + (int64_t)a.id_of[l][i] * a.K;
-    T *z = a.Z[l] + i * a.W;
-    const T v = c < a.C ? Ar[a.S[c]] : T(0);
-    const T p = c >= a.Cq ? T(0) : (a.prev_in_cur ? z[c] : Ar[a.Q[c]]);
-    z[c] = v;
-    z[a.off_old + c] = v;
-    z[CM + c] = p;
+    int l = 0;
+    uint32_t most = 0u;  // of this thread's column in mode l
+    for (int64_t r = (int64_t)blockIdx.x * rows + w; w < rows && r < a.row_base[a.N];
+         r += (int64_t)gridDim.x * rows) {
+        while (r >= a.row_base[l + 1]) {
+            if (a.mx && most) atomicMax(&mx[l * kGateCols + c], most);
+            most = 0u;
+            ++l;
+        }
+        const int64_t i = r - a.row_base[l];  // slice row (rank)
+        const T *Ar = a.A[l] + (int64_t)a.id_of[l][i] * a.K;
+        T *z = a.Z[l] + i * a.W;
+        const T v = c < a.C ? Ar[a.S[c]] : T(0);
+        const T p = c >= a.Cq ? T(0) : (a.prev_in_cur ? z[c] : Ar[a.Q[c]]);
+        z[c] = v;
+        z[a.off_old + c] = v;
+        z[CM + c] = p;
+        if (a.mx) most = max(most, __float_as_uint((float)v) & 0x7FFFFFFFu);
+    }
+    if (!a.mx) return;
+    if (most) atomicMax(&mx[l * kGateCols + c], most);
+    __syncthreads();
+    for (int q = threadIdx.x; q < a.N * kGateCols; q += kPackThreads)
+        record_max(a.mx + q, __uint_as_float(mx[q]));
 }
 
 template <class T>
@@ -386,7 +395,10 @@ template <class T>
 void launch_pack(const PackArgs<T> &a, cudaStream_t st) {
     const int64_t rows = a.row_base[a.N];
     if (rows <= 0) return;
-    k_pack<T><<<blocks_for(rows, kPackThreads / a.off_prev), kPackThreads, 0, st>>>(a);
+    // with maxima few blocks, each over many rows: a block ends with up to N kGateCols atomics
+    unsigned blocks = blocks_for(rows, kPackThreads / a.off_prev);
+    if (a.mx) blocks = std::min(blocks, 1024u);
+    k_pack<T><<<blocks, kPackThreads, 0, st>>>(a);
     TFS_CUDA(cudaGetLastError());
 }
 

@@ -58,33 +58,46 @@ struct PassArgs {
     int refine;
     float cond_limit;
     double *loss_out;  // lean loss pass: per-item (slot) sums of r^2 (other passes: unused)
-    // wide passes of float three-way tensors: bits of the largest |current column value| of the
-    // two other modes (mx), where to record this mode's new one (mx_out; null: nowhere), and
-    // which of two launches of a pass this is (gate: 0 the only one, 1 the one that takes
-    // products in the range of wide_gate, 2 the one that takes the others)
+    // wide passes of float three-way tensors: bits of the largest |value| of every current
+    // column of the two other modes (mx), where to record this mode's new ones (mx_out; null:
+    // nowhere), which of two launches of a pass this is (gate: 0 the only one, 1 the one that
+    // takes products in the range of wide_gate, 2 the one that takes the others), and a count
+    // of the launches that worked (ran)
     const uint32_t *mx[2];
-    uint32_t *mx_out;
+    uint32_t *mx_out, *ran;
     int gate;
     unsigned long long gate_tickets;  // tickets the launch takes in all when it runs
 };
 
+// Columns of a gated sweep's maxima (C <= 63).
+constexpr int kGateCols = 64;
+
 #ifdef __CUDACC__
 // Whether this launch of a gated wide pass is the one that works; the one that does not takes
-// its tickets at once (block 0), which keeps the counter where the host expects it.
+// its tickets at once (block 0), which keeps the counter where the host expects it.  Every
+// column's products have to be zero or large enough for the splits, also of a collapsed column
+// beside healthy ones.  Whole warps.
 template <class T>
 __device__ __forceinline__ bool wide_gate(const PassArgs<T> &a) {
     if (a.gate == 0) return true;
-    const float m0 = __uint_as_float(*a.mx[0]), m1 = __uint_as_float(*a.mx[1]);
-    const double p = (double)m0 * (double)m1;
-    const bool fits = p == 0.0 || (p >= 0x1p-80 && p < 0x1p60);  // NaN: no
-    if (fits == (a.gate == 1)) return true;
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(a.ticket, a.gate_tickets);
-    return false;
+    bool in = true;
+    for (int c = threadIdx.x & 31; c < a.C; c += 32) {
+        const double p = (double)__uint_as_float(a.mx[0][c]) * (double)__uint_as_float(a.mx[1][c]);
+        in = in && (p == 0.0 || (p >= 0x1p-80 && p < 0x1p60));  // NaN: no
+    }
+    const bool fits = __all_sync(0xFFFFFFFFu, in), works = fits == (a.gate == 1);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (works)
+            atomicAdd(a.ran, 1u);
+        else
+            atomicAdd(a.ticket, a.gate_tickets);
+    }
+    return works;
 }
-// Records |v| (bits, one value per lane of the whole warp) as a maximum.
+// Records |v| (bits) as a maximum.
 __device__ __forceinline__ void record_max(uint32_t *slot, float v) {
-    const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(v) & 0x7FFFFFFFu);
-    if ((threadIdx.x & 31) == 0 && m > *(volatile uint32_t *)slot) atomicMax(slot, m);
+    const uint32_t m = __float_as_uint(v) & 0x7FFFFFFFu;
+    if (m > *(volatile uint32_t *)slot) atomicMax(slot, m);
 }
 #endif
 
@@ -97,7 +110,7 @@ struct PackArgs {
     int K, W, C, Cq, off_old, off_prev;
     const int32_t *S, *Q;
     int prev_in_cur;  // the slices' cur regions hold the columns of Q (their final values)
-    uint32_t *mx;     // [N] bits of the largest |cur| value per mode (PassArgs::mx), or null
+    uint32_t *mx;     // [N][kGateCols] bits of the largest |cur| values (PassArgs::mx), or null
     const int32_t *id_of[kMaxModes];  // slice row (rank) -> row id, per mode
 };
 
