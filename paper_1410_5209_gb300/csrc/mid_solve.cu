@@ -92,12 +92,14 @@ __device__ __forceinline__ bool mid_solve(float *P, float *col, int C, float lam
             float d = __shfl_sync(0xFFFFFFFFu, mine, j & 31);
             ok = ok && (d > 0.f);
             d = d > 0.f ? d : 1.f;
-            // quotients by the pivot as products with its inverse and what that leaves (Markstein,
-            // "Computation of elementary functions on the IBM RISC System/6000 processor", IBM
-            // J. Res. Dev. 34, 1990): a rounded inverse alone would scale the whole column
+            // square roots and quotients by fused corrections (Markstein, "Computation of
+            // elementary functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34,
+            // 1990): a quotient is the product with the pivot's inverse and with what that
+            // leaves, since a rounded inverse alone would scale the whole column
             float root, inv;
             if (d > 0x1p-60f && d < 0x1p120f) {
-                // d^1/2 and its inverse from the approximate d^-1/2 by one correction each
+                // d^1/2 and its inverse from the approximate d^-1/2 by one correction each,
+                // where no step leaves the float range
                 inv = rsqrtf(d);
                 root = d * inv;
                 root = fmaf(fmaf(-root, root, d), 0.5f * inv, root);
