@@ -1334,7 +1334,7 @@ struct Impl : CtxBase {
                                     }
                                     a.mx_out = wide_max(s, t + 1, n, T_in);
                                     a.gate = 1;
-                                    a.ran = wide_mx.p;
+                                    a.other_ran = wide_mx.p + (tc ? 2 : 1);
                                     a.gate_tickets = (unsigned long long)L.P +
                                                      (unsigned long long)plan.grid * plan.warps;
                                     timed(TF_KIND_MODE_PASS,
@@ -1342,7 +1342,7 @@ struct Impl : CtxBase {
                                     ticket_base += a.gate_tickets;
                                     a.ticket_base = ticket_base;
                                     a.gate = 2;
-                                    a.ran = wide_mx.p + (tc ? 2 : 1);
+                                    a.other_ran = wide_mx.p;
                                     last_path = kPathGated;
                                     ++launches;
                                 }
