@@ -12,7 +12,7 @@
 //      from shared memory, refreshes its residual copy to this split's R-hat on the
 //      first inner iteration (Algorithm 1; done lazily per copy, see PassArgs) and
 //      accumulates B += h h^T (lower triangle) and c += r_hat h in registers.
-// The warp then sums B and c with butterfly shuffles and writes them to the item's slot.
+// The warp then sums B and c by halving exchanges and writes them to the item's slot.
 // k_solve_rows sums the slots of each row in a fixed order and solves B + lambda I_C (lambda
 // * |Omega_i| when weighted) by a register Cholesky (Section 3.1); the new C parameters go to
 // the packed slice and to A^(n).
