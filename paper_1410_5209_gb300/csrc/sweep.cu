@@ -223,18 +223,18 @@ __global__ void k_init_normal(T *A, int64_t count, uint64_t key, double std) {
 //   The former form, a warp per coordinate with FP64 products and sums, was bound by the
 //   FP64 unit (three conversions, two products and a sum per column at 1/64 of the FP32
 //   rate) and left 22% of its lanes idle at K = 100.  8 lanes per coordinate with 16-byte
-//   loads keep 4 N loads per lane in flight at K = 100.  3,000,017 coordinates, N = 3,
-//   K = 100 on GB300: 6.11 ms before, 0.62 ms now
-//   (5.8 TB/s of gathered rows).
+//   loads take four steps at K = 100.  3,000,017 coordinates, N = 3,
+//   K = 100 on GB300: 6.11 ms before, 0.41 ms now
+//   (8.8 TB/s of gathered rows).
 // A pair loses bits where a product or its error leaves the float range, and a sum of pairs
-// keeps 2^-40 of the terms' magnitudes at worst (Ogita, Rump and Oishi: the square of 2^-24
-// times the additions in a chain; 2^-46 is usual) where FP64 keeps 2^-53.  So a coordinate is
-// formed again in FP64 whose values reach a.big (2^(56 / (N - 1)): no product overflows), whose
-// sum is below 2^-40 or not finite, or whose terms cancel to less than 2^-13 of their
-// magnitudes (below that line the worst error is an eighth of the result's rounding; 1 of 1,000
-// coordinates with terms of random sign, K = 100).  A sum all of whose terms have a zero factor
+// keeps (n 2^-24)^2 of the terms' magnitudes at worst, n additions in a chain (Ogita, Rump and
+// Oishi; 2^-46 is usual), where FP64 keeps 2^-53.  So a coordinate is formed again in FP64 whose
+// values reach a.big (2^(56 / (N - 1)): no product overflows), whose sum is below 2^-40 or not
+// finite, or whose terms' magnitudes are more than a.cancel = 2^21 / n^2 of it: up to there the
+// worst error is an eighth of the result's rounding (n = 10 at K = 100: 3 of 10,000 coordinates
+// with terms of random sign are formed again).  A sum all of whose terms have a zero factor
 // (rows without entries solve to zero) is exact as it is, which a second look at the factors
-// shows where the magnitudes' sum is zero: with 30% of the rows of one mode zero 0.70 ms, and
+// shows where the magnitudes' sum is zero: with 30% of the rows of one mode zero 0.49 ms, and
 // 3.39 when those took the FP64 form too.
 template <class T>
 struct PredictVec;
@@ -247,16 +247,20 @@ struct PredictVec<double> {
     using type = double2;
 };
 
-template <class T, int LP>
-__device__ double predict_f64(const PredictArgs<T> &a, const int32_t *c, int sub, unsigned mask) {
+// One coordinate in FP64 by the whole warp (c the same in every lane): eight lanes took 6 us of
+// a batch of 3,000 for the few coordinates that come here.
+template <class T, int NM>
+__device__ __forceinline__ double predict_f64(const PredictArgs<T> &a, const int32_t *c, int lane) {
+    const int N = NM > 0 ? NM : a.N;
     double s = 0.0;
-    for (int k = sub; k < a.K; k += LP) {
+    for (int k = lane; k < a.K; k += 32) {
         double p = 1.0;
-        for (int n = 0; n < a.N; ++n) p *= (double)a.A[n][(int64_t)c[n] * a.K + k];
+#pragma unroll(NM > 0 ? NM : 1)
+        for (int n = 0; n < N; ++n) p *= (double)a.A[n][(int64_t)c[n] * a.K + k];
         s += p;
     }
 #pragma unroll
-    for (int o = LP / 2; o > 0; o >>= 1) s += __shfl_xor_sync(mask, s, o);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
     return s;
 }
 
@@ -265,27 +269,24 @@ __device__ double predict_f64(const PredictArgs<T> &a, const int32_t *c, int sub
 template <class T, int LP, int NM, bool VEC>
 __global__ void __launch_bounds__(256) k_predict(const PredictArgs<T> a) {
     constexpr int V = VEC ? 16 / (int)sizeof(T) : 1;
-    const int sub = threadIdx.x & (LP - 1);
+    constexpr unsigned kGroup = LP == 32 ? 0xFFFFFFFFu : (1u << LP) - 1u;
+    const int lane = threadIdx.x & 31, sub = lane & (LP - 1), first = lane - sub;
     const int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / LP;
-    if (e >= a.m) return;
-    const unsigned mask = (LP == 32 ? 0xFFFFFFFFu : ((1u << LP) - 1u))
-                          << (threadIdx.x & 31 & ~(LP - 1));
+    const unsigned mask = kGroup << first;
     const int N = NM > 0 ? NM : a.N;
     const int32_t *c = a.coords + e * a.N;
-    bool ok = true;
+    const bool there = e < a.m;
+    bool ok = there;
     const T *row[NM > 0 ? NM : 1];
 #pragma unroll(NM > 0 ? NM : 1)
     for (int n = 0; n < N; ++n) {
-        const int32_t i = c[n];
+        const int32_t i = there ? c[n] : 0;
         ok = ok && i >= 0 && i < a.I[n];
         if (NM > 0) row[NM > 0 ? n : 0] = a.A[n] + (int64_t)i * a.K;
     }
-    if (!ok) {
-        if (sub == 0) {
-            a.out[e] = T(0);
-            atomicOr(&a.stat->bits, kStatPredictRange);
-        }
-        return;
+    if (there && !ok && sub == 0) {
+        a.out[e] = T(0);
+        atomicOr(&a.stat->bits, kStatPredictRange);
     }
     auto load = [&](int n, int k, T (&v)[V]) {
         const T *p = (NM > 0 ? row[NM > 0 ? n : 0] : a.A[n] + (int64_t)c[n] * a.K) + k;
@@ -302,10 +303,14 @@ __global__ void __launch_bounds__(256) k_predict(const PredictArgs<T> a) {
     if constexpr (sizeof(T) == 4) {
         FloatPair sum[V];
         float big = 0.f, mag = 0.f;  // largest factor, sum of the terms' magnitudes
+        const int K = ok ? a.K : 0;
 #pragma unroll
         for (int u = 0; u < V; ++u) sum[u].h = sum[u].l = 0.f;
-#pragma unroll 4
-        for (int k = sub * V; k < a.K; k += LP * V) {
+        // (few steps at once: the other warps hide the loads, and the registers of four steps'
+        // rows leave fewer of them: 3e6 coordinates, K = 100 / 64 / 25: 0.41 / 0.29 / 0.24 ms,
+        // with four steps 0.66 / 0.37 / 0.29)
+#pragma unroll(VEC ? 1 : 2)
+        for (int k = sub * V; k < K; k += LP * V) {
             T v[V];
             FloatPair p[V];
             load(0, k, v);
@@ -337,10 +342,10 @@ __global__ void __launch_bounds__(256) k_predict(const PredictArgs<T> a) {
         for (int o = LP / 2; o > 0; o >>= 1) mag += __shfl_xor_sync(mask, mag, o);
         float r = __fadd_rn(s.h, s.l);
         bool fine = big < a.big && fabsf(r) >= 0x1p-40f && fabsf(r) < 0x1p126f &&
-                    mag <= 0x1p13f * fabsf(r);
+                    mag <= a.cancel * fabsf(r);
         if (mag == 0.f) {  // zero factors, or products that vanished?
             fine = true;
-            for (int k = sub * V; k < a.K; k += LP * V) {
+            for (int k = sub * V; k < K; k += LP * V) {
                 float v[V], least[V];
                 load(0, k, least);
                 for (int n = 1; n < N; ++n) {
@@ -352,10 +357,17 @@ __global__ void __launch_bounds__(256) k_predict(const PredictArgs<T> a) {
                 for (int u = 0; u < V; ++u) fine = fine && least[u] == 0.f;
             }
         }
-        if (__any_sync(mask, !fine)) r = (float)predict_f64<T, LP>(a, c, sub, mask);
-        if (sub == 0) a.out[e] = r;
+        for (unsigned redo = __ballot_sync(0xFFFFFFFFu, !fine); redo;) {
+            const int of = (__ffs(redo) - 1) & ~(LP - 1);  // the first group that asks for it
+            const int64_t er = __shfl_sync(0xFFFFFFFFu, e, of);
+            const double s64 = predict_f64<T, NM>(a, a.coords + er * a.N, lane);
+            if (first == of) r = (float)s64;
+            redo &= ~(kGroup << of);
+        }
+        if (ok && sub == 0) a.out[e] = r;
     } else {
         double s = 0.0;
+        if (!ok) return;
 #pragma unroll 4
         for (int k = sub * V; k < a.K; k += LP * V) {
             T v[V], p[V];
@@ -426,6 +438,10 @@ void launch_predict(const PredictArgs<T> &a, cudaStream_t st) {
     PredictArgs<T> b = a;
     b.big = exp2f(56.f / (float)std::max(a.N - 1, 1));
     if (a.N == 1) b.big = INFINITY;  // no products
+    // additions in a lane's chain, over its vector and over the lanes
+    const int V = a.K % 4 == 0 ? 4 : 1;
+    const float n = (float)((a.K + 8 * V - 1) / (8 * V) + V - 1 + 3);
+    b.cancel = 0x1p21f / (n * n);
     if (a.N == 3)
         launch_predict_lanes<T, 8, 3>(b, st);
     else

@@ -316,7 +316,9 @@ struct PredictArgs {
     const int32_t *coords;
     T *out;
     DeviceStatus *stat;
-    float big;  // float contexts: values from here on take the FP64 form (launch_predict)
+    // float contexts: values from here on, and sums smaller than their terms' magnitudes by
+    // this factor, take the FP64 form (launch_predict)
+    float big, cancel;
 };
 template <class T>
 void launch_predict(const PredictArgs<T> &a, cudaStream_t st);
