@@ -1154,6 +1154,18 @@ struct Impl : CtxBase {
         return kRanWords + (size_t)nsplit * (T_in + 1) * N * kGateCols;
     }
 
+    // The lean pass by default: where its shared-memory cache serves at least a quarter of the
+    // varying mode's gathers (measured slower than the cp.async pass on tensors without hot
+    // rows: a batch of 4,096 small tensors, uniform 1e5^3), and on tensors of up to six default
+    // bins an SM, whose passes are their fixed costs: sweeps of 2,000 to 50,000 entries, five
+    // shapes, C = 2 to 12, 1.0 to 1.4 times as fast as the cp.async pass with nothing cached
+    // (12,000 x 9,000 x 300, 20,000, C = 4: 302 against 411 us), 0.94 to 1.09 at seven bins an
+    // SM, 0.86 to 0.93 at nine.
+    bool lean_pays(const LeanPlan &plan) const {
+        return plan.coverage >= 0.25 ||
+               (lean_cache_rows < 0 && default_bins(num_sms, nnz) <= 6 * num_sms);
+    }
+
     // ------------------------------------------------------------ the sweep
     void sweep(int C, double lambda, int T_in, const int32_t *order, uint32_t flags) {
         if (C < 1 || C > K) throw ApiError{TF_EINVAL, "C must be in 1..K"};
@@ -1396,10 +1408,6 @@ struct Impl : CtxBase {
                             continue;
                         }
                         if constexpr (sizeof(T) == 4) {
-                            // the lean pass where its shared-memory cache serves at
-                            // least a quarter of the varying mode's gathers (measured
-                            // slower than the cp.async pass on tensors without hot rows:
-                            // a batch of 4,096 small tensors, uniform 1e5^3)
                             const std::vector<int64_t> *dc[2] = {&mode[L.omode[0]].deg_cum,
                                                                  &mode[L.omode[1]].deg_cum};
                             const int64_t dims_o[2] = {dims[L.omode[0]], dims[L.omode[1]]};
@@ -1413,7 +1421,7 @@ struct Impl : CtxBase {
                                 plan = lean_pass_plan(CM, t == 0, n, dims_o, dc, nnz, pass_sms(), L.P,
                                                       lean_cache_rows, lean_ring_cap, lean_warps, gk,
                                                       bf16_rows ? precision - 1 : 0);
-                                lean_here = path != 0 || plan.coverage >= 0.25;
+                                lean_here = path != 0 || lean_pays(plan);
                             }
                             if (lean_here) {
                                 const int run = lean_run_mode(n);
@@ -1719,7 +1727,7 @@ struct Impl : CtxBase {
                 // every slot, at two floats or more per slot); the sweep's gather plan must
                 // be kept (the loss builds and allocates nothing)
                 const int run0 = lean_run_mode(0);
-                lean_loss = (path != 0 || lplan.coverage >= 0.25) && partials.p != nullptr &&
+                lean_loss = (path != 0 || lean_pays(lplan)) && partials.p != nullptr &&
                             partials.n >= (size_t)2 * (size_t)std::max<int64_t>(L.n_slots, 1) &&
                             find_gather_plan(0, lplan.p.R[run0], lplan.p.R[1 - run0],
                                              lplan.p.cap[0]) != nullptr;

@@ -734,7 +734,7 @@ LeanPlan lean_pass_plan(int CM, bool first, int n, const int64_t *dims_o,
     // what the cache serves, which decides between this pass and the staged one: rows that are
     // not worth their copies leave nothing here (three passes of 700^3, 1e5 entries, C = 4 / 10:
     // 16.3 / 22.8 us each with empty caches, 13.3 / 14.9 in the staged pass; 12,000^3, 1.6e6,
-    // C = 4: 54 and 45; the other way only below 5e4 entries, 3,000^3, 4e4: 11.5 and 14.3)
+    // C = 4: 54 and 45)
     {
         const int var = 1 - lean_run_mode(n);
         const std::vector<int64_t> &dc = *deg_cum[var];
