@@ -36,9 +36,9 @@ WORKLOAD = dict(workload="skewed_3way_1e8", dims=[100_000, 100_000, 1_000], nnz=
 # profiles/k_lean_pass_skewed_3way_1e8.md (2e7-entry case, scaled by entries to a
 # 1e8-entry launch), and the hash of the kernel sources it was taken with; the bench
 # reports traffic as null once the sources differ or the entry count is not 1e8.
-NCU_TRAFFIC = 1.690e9
+NCU_TRAFFIC = 1.689e9
 NCU_TRAFFIC_NNZ = 100_000_000
-NCU_SOURCE_HASH = "4573899abf969c28"
+NCU_SOURCE_HASH = "4447a128fba5b8d5"
 
 
 # Utilisation of the L1 data pipe (shared-memory and L1 wavefronts) of the mode pass in the
