@@ -130,6 +130,12 @@ __device__ __forceinline__ bool chol_factor(T (&B)[CM * (CM + 1) / 2], T (&inv)[
     // the matrix of CM = 6 and 8 in local memory)
 #pragma unroll
     for (int j = 0; j < CM; ++j) {
+        // double: nothing to do for the identity's rows (a root, a division and their products
+        // on a unit that takes 64 cycles a step; 1,000 rows, C = 5: 21 us, 19.5 without them)
+        if (sizeof(T) == 8 && j >= C) {
+            inv[j] = T(1);
+            continue;
+        }
         const T a_jj = B[tri(j, j)];
         T d = a_jj;
 #pragma unroll
@@ -142,7 +148,7 @@ __device__ __forceinline__ bool chol_factor(T (&B)[CM * (CM + 1) / 2], T (&inv)[
         inv[j] = sizeof(T) == 8 ? T(1) / piv : T(0);
 #pragma unroll
         for (int i = 0; i < CM; ++i) {
-            if (i <= j) continue;
+            if (i <= j || (sizeof(T) == 8 && i >= C)) continue;
             T s = B[tri(i, j)];
 #pragma unroll
             for (int k = 0; k < CM; ++k)
@@ -963,7 +969,7 @@ __global__ void __launch_bounds__(kOneWarps * kWarp, 1) k_pass_one(const PassArg
 // solved the single-slot rows, each thread reading its row's slot at a stride of NB values,
 // and a second took 512 threads per split row: 44 + 55 us per mode of 1e5 rows (1e8 entries,
 // C = 10), now 61; 1,000 FP64 rows of two slots, C = 5: 127 us (a lone lane's FP64
-// instructions take the unit as long as a full warp's), now 19.
+// instructions take the unit as long as a full warp's), now 19.5.
 // XS: the solve options of float contexts (refinement / FP64 fallback) are on; the plain
 // Cholesky otherwise, so that the default kernels carry none of their registers.
 template <class T, int CM, bool XS>
