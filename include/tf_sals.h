@@ -263,18 +263,21 @@ tf_status tf_foldin(tf_ctx *ctx, int mode, const int32_t *other, const void *val
  *   device buffers on the context's device with flags = TF_INPUT_DEVICE.
  * Products and the sum over k in double on the device, in float contexts in pairs of floats
  * (about 48 bits) where the terms' range and cancellation leave a float result the same
- * accuracy.  Synchronises.  TF_ERANGE if a
- * coordinate is out of range (out is then unspecified). */
+ * accuracy.  Synchronises.  TF_ERANGE if a coordinate is out of range (out is then
+ * unspecified). */
 tf_status tf_predict(tf_ctx *ctx, const int32_t *coords, int64_t m, void *out, uint32_t flags);
 
-/* Many fold-in requests of one mode in one batch (one launch of the tiled Gram over all
- * of their entries, one warp-level solve per request): request r has the entries
+/* Many fold-in requests of one mode in one batch (blocks over the entries of all requests,
+ * the last block of each solves it): request r has the entries
  * offsets[r] .. offsets[r + 1] - 1 of the concatenated other [total][N-1] and values
  * [total] (host; offsets[n_req + 1] int64 with offsets[0] = 0, non-decreasing).
  * out_rows [n_req][K] (host, context dtype); status [n_req] (host): 0 ok, 1 an index
  * out of range, 2 a non-positive pivot — the row of a failed request is left untouched
  * and the others are still solved.  Synchronises.  Results equal tf_foldin's per
- * request (same blocks, same summation order). */
+ * request (same blocks, same summation order).  Device scratch beside the requests and
+ * rows: 64 MiB, or what the largest request needs (a partial system, 23 KB at K = 100 and
+ * twice that in double, for every 64 entries up to 1,024, every 256 beyond), kept by the
+ * context. */
 tf_status tf_foldin_batch(tf_ctx *ctx, int mode, int n_req, const int64_t *offsets,
                           const int32_t *other, const void *values, double lambda, void *out_rows,
                           int32_t *status);
