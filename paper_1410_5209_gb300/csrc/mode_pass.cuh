@@ -1211,7 +1211,9 @@ struct ResConsumer {
     __device__ __forceinline__ void item_end(const Step &, int) {}
 };
 
-// Number of other modes as a compile-time constant: five-way float tensors, any (0).
+// Number of other modes as a compile-time constant: five-way float tensors, any (0).  Orders 4 and
+// 6 to 8 and double run the generic kernel; the constant, the 16-byte windows and the single row
+// slot were not measured for them.
 template <class T>
 __host__ __device__ constexpr int res_no(int N) {
     return sizeof(T) == 4 && N == 5 ? 4 : 0;
